@@ -21,6 +21,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "project.cuh"
 
 namespace mgct {
 
@@ -32,7 +33,8 @@ struct BPArgs {
     int n, nu, nv;
     float h;
     int view0, stride, nviews;
-    int splits;  // slab kernel: view ranges per z-slab, each into its own partial volume (1: none)
+    int splits;  // plane kernel: view ranges, each into its own partial volume (1: none)
+    int cls;     // plane kernel: the ray class (1: y-major), or -1 for both in one launch
 };
 
 template <int NCH, typename ST>
@@ -51,10 +53,6 @@ struct SinoLoad<2, float2> {
         acc[1] = fmaf(w, y.y, acc[1]);
     }
 };
-
-__device__ __forceinline__ float2 load_f2(const float2 *p) { return __ldg(p); }
-template <typename ST>
-__device__ __forceinline__ float2 load_f2(const ST *) { return make_float2(0.0f, 0.0f); }
 
 // Adds A^T (one view) at voxel (jx, jy, jz) into acc -- any geometry.
 // WEIGHTED: the sinogram already carries each ray's dl (see the projector's
@@ -146,8 +144,8 @@ __device__ __forceinline__ void bp_view_sep(const ViewGeom &G, const float4 *__r
     const float cx = (float)jx - ic, cy = (float)jy - ic;
     const float zm = (float)jz0 - ic + 0.5f * (float)(ZB - 1);  // centre of the thread's voxels (exact)
     for (int ju = ulo; ju <= uhi; ++ju) {
-        const float4 t0 = __ldg(cols + 4 * ju), t1 = __ldg(cols + 4 * ju + 1);
-        const float4 t2 = __ldg(cols + 4 * ju + 2), t3 = __ldg(cols + 4 * ju + 3);
+        const float4 t0 = __ldg(cols + ju), t1 = __ldg(cols + a.nu + ju);
+        const float4 t2 = __ldg(cols + 2 * a.nu + ju), t3 = __ldg(cols + 3 * a.nu + ju);
         const bool ay = t0.x != 0.0f;
         const float ca = ay ? cy : cx, cb = ay ? cx : cy;
         const DF eb = df_add(df_mul_f(DF{t0.y, t0.z}, ca), DF{t0.w, t1.x});
@@ -272,178 +270,407 @@ __global__ void __launch_bounds__(BP_BX *BP_BY *BP_BZ)
     }
 }
 
-// Separable geometry, weighted sinogram: the solver's hot path.
-// Each thread owns one (x, y) voxel column and a slab of Z voxels along z,
-// accumulated in shared memory.  Per view and per detector column u' whose
-// rays meet the voxel column (|e_b| < 1), the z crossing of the ray through
-// pixel (u', v') is f_z(v') = E0' + v' E1 (E0' uncentred), so the voxels the
-// ray touches are floor(f_z) and floor(f_z) + 1 with weights (1 - t, t),
-// t = f_z - floor(f_z): the exact transpose of the projector's bilinear tap
-// in z.  Each pixel of the slab's v range is visited once and splatted into
-// the thread's own shared-memory column (no two threads share a column, so
-// no atomics, and the order of additions is fixed).  Lanes are adjacent x
-// columns, so the pixel reads of a warp fall on one detector row.
-constexpr int BS_TX = 32, BS_TY = 4, BS_THREADS = BS_TX * BS_TY;
-constexpr float BS_MAGIC = 12582912.0f;  // 1.5 * 2^23
-constexpr int BS_MAGIC_BITS = 0x4B400000;
+// Separable geometries, weighted sinogram stored [view][u][v] (rows
+// contiguous) with SINO_PAD zero rows before and after every column: the
+// solver's A^T and, after k_weight_rays, the public one.
+//
+// A warp owns W voxel columns of one voxel-centre plane -- consecutive along
+// the plane's in-plane axis b -- over ZT heights, its lanes the heights (lane
+// l: z0 + l, z0 + 32 + l, ...).  The rays of one detector column cross the
+// plane at one in-plane position b, so the column's z profile there,
+//   g(z) = sum over rows of y hat(f_z(row) - z),
+// is computed once, by all lanes together, and added with the weights
+// (1 - t_b, t_b) to the two voxel columns jb and jb + 1 it falls between: no
+// lane waits for another's columns, and the rows a warp reads are one
+// contiguous run.  Columns of y-major rays take the planes y = const, those
+// of x-major rays the planes x = const, in blocks of their own (two partial
+// volumes added afterwards, or two launches where there is no room for them).
+//
+// Detector columns are taken 32 at a time, across views, a lane per column:
+// the lane sets up everything that depends on (view, plane, column) alone, in
+// double-float, and the warp sorts the 32 by jb (counting sort) into a table
+// that the profile loop reads by broadcast.  The two voxel columns of the
+// current jb stay in registers; the tile's others in shared memory.
+//
+// The row heights are anchored at the detector row nearest the tile's middle
+// height and formed with one rounding each (ri E - z exactly fused), so a
+// weight is accurate to ~1e-7 at any N.  Lane z's rows start at
+// ri = ceil((z - 1 - E0) / E): that row's weight is its height above z - 1,
+// the following ones' 1 - |height - z|, as long as the height stays below
+// z + 1 (rows beyond are not loaded).
+//
+// Bound by issue slots and L1 wavefronts alike (profile at 256^3 / 144 views:
+// 69 % issue-active, 73 % L1; 34 instructions and 9 wavefronts per column,
+// plane and 32 heights, of which the profile's 3 or 4 row loads are 6
+// wavefronts).  A thread per voxel column, as before, computed every profile
+// twice, at 68 instructions, with lanes waiting for each other's columns.
+constexpr int BT_WARPS = 8;   // planes per block
+constexpr float BT_MAGIC = 12582912.0f;  // 1.5 * 2^23: ceil(x) in the low mantissa bits of x + BT_MAGIC rounded up
+constexpr int BT_MAGIC_BITS = 0x4B400000;
 
-#ifndef MGCT_BS_PAIRS
-#define MGCT_BS_PAIRS 1
-#endif
-#ifndef MGCT_BS_REG
-#define MGCT_BS_REG 1
-#endif
-template <int NCH>
-struct SlabCfg {
-    // voxels per slab: 16 keeps the shared slab at 10 KB so that 16 blocks
-    // (64 warps) fit per SM; measured 64 -> 32 -> 16: 74 -> 63 -> 55 ms per
-    // grid-0 launch at 256^3 / 720 views
-    static constexpr int Z = 16 / NCH;
-    static constexpr int ROWS = Z + 5;  // guard rows: two below, three above (row pairs reach r + 2)
+// One detector column at one plane.  The rows of a height zl above the tile's
+// middle start at ceil(fma(zl, rE, -d1 rE)), counted from the anchor row.
+struct __align__(16) ColEntry {
+    float E, Elo;     // E + Elo: height step per row
+    float d1, rE;     // 1 + height of the anchor row; 1 / E
+    long long base;   // element of the anchor row in the sinogram, less BT_MAGIC_BITS
+    float tb;         // fraction along b
+    float rlo;        // the first readable row, -SINO_PAD, from the anchor, plus BT_MAGIC
 };
 
-// DFA = true: the public A^T at any N.  The column comes from the double-
-// float table and its z crossing is anchored, in double-float, at the detector
-// row nearest the slab's centre, so the crossings are stepped in float32 from
-// a small height relative to the slab (accurate to ~1e-6 voxel at any N; the
-// float32 table's uncentred heights near z = 1000 carry ~6e-5).
-template <int NCH, typename ST, bool DFA = false>
-__global__ void __launch_bounds__(BS_THREADS)
-    k_backproject_slab(BPArgs a, const float4 *__restrict__ cols, const ST *__restrict__ sino,
-                       float *__restrict__ out, int accumulate) {
-    constexpr int Z = SlabCfg<NCH>::Z, ROWS = SlabCfg<NCH>::ROWS;
-    constexpr int CW = DFA ? 4 : 2;  // float4 per table entry
-    __shared__ float acc[NCH][ROWS][BS_THREADS];
-    const int tid = threadIdx.x;
-    const int jx = blockIdx.x * BS_TX + (tid % BS_TX), jy = blockIdx.y * BS_TY + tid / BS_TX;
-    // blockIdx.z = split * (z-slabs) + slab; split s takes views [i0, i1)
-    // and writes partial volume s of `out`
-    const int splits = DFA ? 1 : a.splits;  // the public form never splits
-    const int zblocks = gridDim.z / splits;
-    const int split = blockIdx.z / zblocks;
-    const int z0 = (blockIdx.z - split * zblocks) * Z;
-    const int per = (a.nviews + splits - 1) / splits;
-    const int i0 = split * per, i1 = min(a.nviews, i0 + per);
-#pragma unroll
-    for (int q = 0; q < NCH; ++q)
-        for (int r = 0; r < ROWS; ++r) acc[q][r][tid] = 0.0f;
-    if (jx < a.n && jy < a.n) {
-        const float ic = 0.5f * (float)(a.n - 1);
-        const float cu = 0.5f * (float)(a.nu - 1), cv = 0.5f * (float)(a.nv - 1);
-        const float cx = (float)jx - ic, cy = (float)jy - ic;
-        const float zlo = (float)z0 - 1.0f, zhi = (float)(z0 + Z);  // crossings that touch the slab
-        const size_t view_elems = (size_t)a.nu * a.nv;
-        for (int i = i0; i < i1; ++i) {
-            const int k = a.view0 + i * a.stride;
-            const float *G = reinterpret_cast<const float *>(a.views + k);
-            // projected u range of the voxel column (the cube bound; z-free without tilt)
-            const float X = (float)jx - __ldg(G + 0), Y = (float)jy - __ldg(G + 1);
-            const float Q0 = __ldg(G + 12), Q1 = __ldg(G + 13), Q6 = __ldg(G + 18), Q7 = __ldg(G + 19);
-            const float q2 = fmaf(Q7, Y, Q6 * X);
-            const float u0 = fmaf(Q1, Y, Q0 * X) * __frcp_rn(q2);
-            const float hu = (fabsf(Q0 - u0 * Q6) + fabsf(Q1 - u0 * Q7)) * __frcp_rn(q2 - __ldg(G + 21));
-            const int ulo = max(0, (int)ceilf(u0 - hu + cu - 1e-3f));
-            const int uhi = min(a.nu - 1, (int)floorf(u0 + hu + cu + 1e-3f));
-            const ST *__restrict__ sv = sino + (size_t)i * view_elems;
-            const float4 *__restrict__ ct = cols + (size_t)k * a.nu * CW;
-            for (int ju = ulo; ju <= uhi; ++ju) {
-                const float4 t0 = __ldg(ct + CW * ju);
-                const float4 t1 = __ldg(ct + CW * ju + 1);
-                const bool ay = t0.x != 0.0f;
-                const float ca = ay ? cy : cx, cb = ay ? cx : cy;
-                // E0, E1: crossing height at row offset vf = 0 and its slope per
-                // row; zb: the height E0 is counted from (uncentred z)
-                float hb, E0, E1, vf;
-                int vlo, vhi, zb;
-                if constexpr (!DFA) {
-                    hb = 1.0f - fabsf(fmaf(ca, t0.y, t0.z) - cb);
-                    if (hb <= 0.0f) continue;
-                    E0 = fmaf(ca, t1.x, t0.w) + ic;  // uncentred z crossing at v' = 0
-                    E1 = fmaf(ca, t1.z, t1.y);
-                    const float rE = __frcp_rn(E1);
-                    const float ta = fmaf(zlo - E0, rE, cv), tb = fmaf(zhi - E0, rE, cv);
-                    vlo = max(0, (int)ceilf(fminf(ta, tb) - 1e-3f));
-                    vhi = min(a.nv - 1, (int)floorf(fmaxf(ta, tb) + 1e-3f));
-                    vf = (float)vlo - cv;
-                    zb = z0;
-                } else {
-                    const float4 t2 = __ldg(ct + CW * ju + 2), t3 = __ldg(ct + CW * ju + 3);
-                    const DF eb = df_add(df_mul_f(DF{t0.y, t0.z}, ca), DF{t0.w, t1.x});
-                    hb = 1.0f - fabsf(__fadd_rn(__fsub_rn(eb.hi, cb), eb.lo));
-                    if (hb <= 0.0f) continue;
-                    const DF Eb = df_add(DF{t1.y, t1.z}, df_mul_f(DF{t1.w, t2.x}, ca));   // centred, v' = 0
-                    const DF E1d = df_add(DF{t2.y, t2.z}, df_mul_f(DF{t2.w, t3.x}, ca));
-                    E1 = E1d.hi;
-                    const float zc = (float)z0 - ic + 0.5f * (float)(Z - 1);  // slab centre, centred (exact)
-                    const float va = rintf((zc - Eb.hi) / E1);                // anchor row, centred v'
-                    if (!(fabsf(va) < 1.0e7f)) continue;
-                    const DF c = df_add(df_add(Eb, df_mul_f(E1d, va)), DF{-zc, 0.0f});
-                    E0 = (c.hi + c.lo) + 0.5f * (float)(Z - 1);  // height above z0 at the anchor row
-                    const float rE = __frcp_rn(E1);
-                    const float ta = fmaf(-1.0f - E0, rE, va + cv), tb = fmaf((float)Z - E0, rE, va + cv);
-                    vlo = max(0, (int)ceilf(fminf(ta, tb) - 1e-3f));
-                    vhi = min(a.nv - 1, (int)floorf(fmaxf(ta, tb) + 1e-3f));
-                    vf = ((float)vlo - cv) - va;  // rows from the anchor (exact)
-                    zb = 0;
-                }
-                const ST *__restrict__ px = sv + (size_t)vlo * a.nu + ju;
-                int jv = vlo;
-                if constexpr (NCH == 1) {
-                  if (MGCT_BS_PAIRS && E1 > 0.0f && E1 < 0.999f) {
-                    // two rows at a time: their crossings floor(fz) are equal or
-                    // one apart (0 < E1 < 1), so the pair touches three slab
-                    // rows r, r + 1, r + 2 -- three read-modify-writes, not four
-                    // floor(fz) from one addition rounded toward minus infinity
-                    // (fz + 1.5 * 2^23 holds it in its low mantissa bits); a
-                    // row index outside the slab wraps, as unsigned, to the top
-                    // guard rows
-                    const int rbase = BS_MAGIC_BITS + zb - 2;
-                    for (; jv + 1 <= vhi; jv += 2, vf += 2.0f, px += 2 * (size_t)a.nu) {
-                        const float fz0 = fmaf(vf, E1, E0), fz1 = fmaf(vf + 1.0f, E1, E0);
-                        const float m0 = __fadd_rd(fz0, BS_MAGIC), m1 = __fadd_rd(fz1, BS_MAGIC);
-                        const float t0 = fz0 - (m0 - BS_MAGIC), t1 = fz1 - (m1 - BS_MAGIC);
-                        const int r = (int)min((unsigned)(__float_as_int(m0) - rbase), (unsigned)(ROWS - 3));
-                        const bool same = __float_as_int(m1) == __float_as_int(m0);
-                        const float y0 = hb * to_f32(__ldg(px)), y1 = hb * to_f32(__ldg(px + a.nu));
-                        const float a0 = y0 * t0, b0 = y1 * t1;
-                        const float lo1 = y1 - b0;
-                        acc[0][r][tid] += (y0 - a0) + (same ? lo1 : 0.0f);
-                        acc[0][r + 1][tid] += a0 + (same ? b0 : lo1);
-                        if (!same) acc[0][r + 2][tid] += b0;
-                    }
-                  }
-                }
-                for (; jv <= vhi; ++jv, vf += 1.0f, px += a.nu) {
-                    const float fz = fmaf(vf, E1, E0);
-                    const float fl = floorf(fz);
-                    const float t = fz - fl;
-                    // row of voxel floor(fz) in the guarded slab: in [0, Z + 2]
-                    const int r = min(max((int)fl - zb + 2, 0), ROWS - 2);
-                    if constexpr (NCH == 1) {
-                        const float yw = hb * to_f32(__ldg(px));
-                        const float w1 = yw * t;
-                        acc[0][r][tid] += yw - w1;
-                        acc[0][r + 1][tid] += w1;
-                    } else {
-                        const float2 y2 = load_f2(px);
-                        const float ya = hb * y2.x, yb = hb * y2.y;
-                        acc[0][r][tid] += ya - ya * t;
-                        acc[0][r + 1][tid] += ya * t;
-                        acc[NCH - 1][r][tid] += yb - yb * t;
-                        acc[NCH - 1][r + 1][tid] += yb * t;
-                    }
-                }
-            }
+// NP: pairs of values a lane holds, two heights of one channel or the two
+// channels of one height; W: voxel columns per warp.  Measured, public call at
+// 256^3 / 720 views: W = 8 with two pairs and 24 resident warps, or one pair
+// and 32, 22.0 ms; one pair and 24 warps 23.9; 16 columns with two pairs 25.6
+// (its accumulators leave half the L1), with one 23.4; the slab kernel that
+// this one replaced 52.0, the solver's register kernel 29.5 (22.0 here).
+template <int NCH, int NP>
+struct PlaneTile {
+    static constexpr int ZT = NCH == 2 ? 32 * NP : 64 * NP, ZP = ZT + 1;
+    static constexpr int W = 8;
+    static constexpr int MIN_BLOCKS = NP == 2 ? 3 : 4;  // 80 and 64 registers
+    static constexpr size_t acc_floats = (size_t)BT_WARPS * W * NCH * ZP;
+    static constexpr size_t smem = sizeof(ColEntry) * 32 * BT_WARPS + sizeof(float) * acc_floats;
+};
+
+// packed float pairs (one instruction each)
+__device__ __forceinline__ float2 add_f2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 add_up_f2(float2 a, float2 b) {  // rounded toward plus infinity
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "add.rp.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 mul_f2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "mul.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
+
+// A load where `w` is positive, 0 elsewhere (nothing read).
+__device__ __forceinline__ float ld_if(const float *p, float w) {
+    float v;
+    asm("{\n\t.reg .pred q;\n\tsetp.gt.f32 q, %2, 0f00000000;\n\tmov.f32 %0, 0f00000000;\n\t"
+        "@q ld.global.nc.f32 %0, [%1];\n\t}"
+        : "=f"(v)
+        : "l"(p), "f"(w));
+    return v;
+}
+// Row s of a lane's pair, with (w) or without a weight that has to be positive.
+__device__ __forceinline__ float2 bt_row(const float *pa, const float *pb, int s) {
+    return make_float2(__ldg(pa + s), __ldg(pb + s));
+}
+__device__ __forceinline__ float2 bt_row(const float2 *pa, const float2 *, int s) { return __ldg(pa + s); }
+__device__ __forceinline__ float2 bt_row(const float *pa, const float *pb, int s, float2 w) {
+    return make_float2(ld_if(pa + s, w.x), ld_if(pb + s, w.y));
+}
+__device__ __forceinline__ float2 bt_row(const float2 *pa, const float2 *, int s, float2 w) {
+    float2 v;
+    asm("{\n\t.reg .pred q;\n\tsetp.gt.f32 q, %3, 0f00000000;\n\tmov.f32 %0, 0f00000000;\n\tmov.f32 %1, 0f00000000;\n\t"
+        "@q ld.global.nc.v2.f32 {%0, %1}, [%2];\n\t}"
+        : "=f"(v.x), "=f"(v.y)
+        : "l"(pa + s), "f"(w.x));
+    return v;
+}
+
+// Profile at one height of any column, rows off the detector reading as zero;
+// v: the height's first row, col: the column's row 0.
+template <typename ST>
+__device__ __forceinline__ float2 bt_profile_any(const ST *__restrict__ col, int v, int nv, float g, float E) {
+    float2 a = make_float2(0.0f, 0.0f);
+    for (int s = 0; v < nv; ++s, ++v) {
+        const float h = fmaf((float)s, E, g) - 1.0f;
+        if (!(h < 1.0f)) break;
+        if (v < 0) continue;
+        a = fma_f2(both(1.0f - fabsf(h)), bt_row(col, col, v), a);
+    }
+    return a;
+}
+
+// First row m of a pair of heights zl, as a number at BT_MAGIC, and 1 + (its
+// height - zl).
+__device__ __forceinline__ float2 bt_start(const ColEntry &t, float2 zl, float2 &m) {
+    m = add_up_f2(fma_f2(zl, both(t.rE), both(-t.d1 * t.rE)), both(BT_MAGIC));
+    const float2 ri = add_f2(m, both(-BT_MAGIC));
+    return add_f2(fma_f2(ri, both(t.E), make_float2(-zl.x, -zl.y)), fma_f2(ri, both(t.Elo), both(t.d1)));
+}
+
+// Profile of table entry t at the pair zl of heights from ROWS rows: 3 or 4
+// where 2/3 < E < 1 or 1/2 < E < 1, 5 for any E > 0.4.  Rows off the detector
+// are the sinogram's zero rows: a start is clamped to those before and after
+// the column, without a change of the weights.
+template <int ROWS, int NCH, typename ST>
+__device__ __forceinline__ float2 bt_profile(const ColEntry &t, const ST *__restrict__ anchor, float rspan, float2 zl) {
+    // a second channel takes the first one's weights
+    auto pair = [](float2 w) { return NCH == 2 ? make_float2(w.x, w.x) : w; };
+    float2 m;
+    const float2 g = bt_start(t, zl, m);
+    const float rhi = t.rlo + rspan;
+    const ST *pa = anchor + __float_as_int(fminf(fmaxf(m.x, t.rlo), rhi));
+    const ST *pb = anchor + __float_as_int(fminf(fmaxf(m.y, t.rlo), rhi));
+    if (ROWS < 5) {
+        // the first two rows lie below z + 1 whatever g (g < E < 1); from the
+        // third on the height is above z (2 E > 1)
+        const float2 h1 = add_f2(g, both(t.E - 1.0f));
+        const float2 w1 = make_float2(1.0f - fabsf(h1.x), 1.0f - fabsf(h1.y));
+        const float2 w2 = fma_f2(g, both(-1.0f), both(fmaf(-2.0f, t.E, 2.0f)));
+        const float2 y0 = bt_row(pa, pb, 0), y1 = bt_row(pa, pb, 1), y2 = bt_row(pa, pb, 2, w2);
+        float2 p = mul_f2(pair(g), y0);
+        if (ROWS == 4) {
+            const float2 w3 = fma_f2(g, both(-1.0f), both(fmaf(-3.0f, t.E, 2.0f)));
+            p = fma_f2(pair(w3), bt_row(pa, pb, 3, w3), p);
         }
-        const size_t nvox = (size_t)a.n * a.n * a.n;
-        float *o = out + (size_t)split * NCH * nvox;
-        for (int zz = 0; zz < Z; ++zz) {
-            const int z = z0 + zz;
-            if (z >= a.n) break;
-            const size_t idx = ((size_t)z * a.n + jy) * a.n + jx;
+        p = fma_f2(pair(w1), y1, p);
+        return fma_f2(pair(w2), y2, p);
+    }
+    float2 h = add_f2(g, both(-1.0f)), p = both(0.0f);
+#pragma unroll
+    for (int s = 0; s < ROWS; ++s) {
+        const float2 w = make_float2(1.0f - fabsf(h.x), 1.0f - fabsf(h.y));
+        // beyond the second row often no lane has any (E >= 1)
+        if (s < 2 || __any_sync(0xffffffffu, fmaxf(w.x, w.y) > 0.0f)) p = fma_f2(pair(w), bt_row(pa, pb, s, w), p);
+        h = add_f2(h, both(t.E));
+    }
+    return p;
+}
+
+// The same for any E, row by row; nv: the detector's rows.
+template <int NCH, typename ST>
+__device__ __forceinline__ float2 bt_profile_loop(const ColEntry &t, const ST *__restrict__ anchor, int nv, float2 zl) {
+    float2 m;
+    const float2 g = bt_start(t, zl, m);
+    const int row0 = __float_as_int(t.rlo) + SINO_PAD;  // the detector's row 0, as the rows' bits
+    const ST *col = anchor + row0;
+    float2 p = bt_profile_any(col, __float_as_int(m.x) - row0, nv, g.x, t.E);
+    if (NCH == 1) p.y = bt_profile_any(col, __float_as_int(m.y) - row0, nv, g.y, t.E).x;
+    return p;
+}
+
+template <int NCH, int NP, typename ST>
+__global__ void __launch_bounds__(32 * BT_WARPS, PlaneTile<NCH, NP>::MIN_BLOCKS)
+    k_backproject_plane(BPArgs a, const float4 *__restrict__ cols, const int2 *__restrict__ ranges,
+                        const ST *__restrict__ sino, float *__restrict__ out, int accumulate) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    using T = PlaneTile<NCH, NP>;
+    constexpr int ZT = T::ZT, ZP = T::ZP, W = T::W;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    ColEntry *tab = reinterpret_cast<ColEntry *>(smem_raw) + 32 * warp;
+    float *acc = reinterpret_cast<float *>(smem_raw + sizeof(ColEntry) * 32 * BT_WARPS);  // [warp][W][NCH][ZP]
+    // blockIdx.z = part * (z tiles) + tile; part = class * splits + split where
+    // both classes run in one launch; split s takes views [i0, i1), and part q
+    // writes partial volume q of `out`
+    const int parts = a.splits * (a.cls < 0 ? 2 : 1);
+    const int ztiles = gridDim.z / parts;
+    const int part = blockIdx.z / ztiles;
+    const int z0 = (blockIdx.z - part * ztiles) * ZT;
+    const int cls = a.cls < 0 ? part / a.splits : a.cls;
+    const int split = part - (a.cls < 0 ? cls * a.splits : 0);
+    const int per = (a.nviews + a.splits - 1) / a.splits;
+    const int i0 = split * per, i1 = min(a.nviews, i0 + per);
+    // this warp's plane (of axis y for class 1, x for class 0), the tile's first
+    // voxel along b and its width
+    const int p0 = blockIdx.y * BT_WARPS, pl = p0 + warp, b0 = blockIdx.x * W;
+    const int wb = min(W, a.n - b0);
+    const float ic = 0.5f * (float)(a.n - 1);
+    const float cu = 0.5f * (float)(a.nu - 1), cv = 0.5f * (float)(a.nv - 1);
+    const float ca = (float)pl - ic, cb0 = (float)b0 - ic;
+    const float zc = (float)(z0 + ZT / 2) - ic;  // the tile's middle height, centred (exact)
+    float2 zl[NP];
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+        const float z = (float)(lane - ZT / 2 + i * (ZT / NP));
+        zl[i] = make_float2(z, NCH == 2 ? z : z + 32.0f);
+    }
+    const float rspan = (float)(a.nv + SINO_PAD);  // from the first to the last readable start
+    for (int t = tid; t < (int)T::acc_floats; t += 32 * BT_WARPS) acc[t] = 0.0f;
+    __syncthreads();
+    float *const accw = acc + warp * W * NCH * ZP + lane;
+
+    for (int ib = i0; ib < i1 && pl < a.n; ib += 32) {
+        // lane = view: the detector columns of this class whose rays cross the
+        // plane strictly between voxels b0 - 1 and b0 + wb, i.e. between the
+        // projections of those two points (with a margin far above their
+        // rounding; the exact test is the column's own)
+        int vlo = 0, cnt = 0;
+        if (ib + lane < i1) {
+            const int k = a.view0 + (ib + lane) * a.stride;
+            const float *G = reinterpret_cast<const float *>(a.views + k);
+            const float Sx = __ldg(G + 0), Sy = __ldg(G + 1);
+            const float Q0 = __ldg(G + 12), Q1 = __ldg(G + 13), Q6 = __ldg(G + 18), Q7 = __ldg(G + 19);
+            const float Xa = (float)(cls ? b0 - 1 : pl) - Sx, Ya = (float)(cls ? pl : b0 - 1) - Sy;
+            const float db = (float)(wb + 1);
+            const float qa0 = fmaf(Q1, Ya, Q0 * Xa), qa2 = fmaf(Q7, Ya, Q6 * Xa);
+            const float qb0 = fmaf(cls ? Q0 : Q1, db, qa0), qb2 = fmaf(cls ? Q6 : Q7, db, qa2);
+            const float ua = qa0 / qa2 + cu, ub = qb0 / qb2 + cu;
+            const int2 r = __ldg(ranges + 2 * k + cls);
+            vlo = max(r.x, (int)ceilf(fminf(ua, ub) - 1e-2f));
+            cnt = max(0, min(r.y, (int)floorf(fmaxf(ua, ub) + 1e-2f)) - vlo + 1);
+        }
+        // inclusive prefix sums: the views' columns as one list of `total`
+        int pre = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(FULL, pre, o);
+            if (lane >= o) pre += v;
+        }
+        const int total = __shfl_sync(FULL, pre, 31);
+        for (int first = 0; __any_sync(FULL, first < total); first += 32) {
+            // lane = column `first + lane` of the list: its view is the number
+            // of views that end at or before it
+            const int idx = first + lane;
+            int v = 0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(FULL, pre, v + o - 1) <= idx) v += o;
+            const int ju = __shfl_sync(FULL, vlo, v & 31) + idx - __shfl_sync(FULL, pre - cnt, v & 31);
+            const int i = ib + v;
+            int jb = -2;  // not in the tile
+            int rows = 0, on = 0;  // rows of a height (0: any number), pairs of heights with rows on the detector
+            ColEntry te;
+            if (idx < total) {
+                const float4 *c = cols + (size_t)(a.view0 + i * a.stride) * 4 * a.nu + ju;
+                const float4 t0 = __ldg(c), t1 = __ldg(c + a.nu), t2 = __ldg(c + 2 * a.nu), t3 = __ldg(c + 3 * a.nu);
+                const DF rb{t0.y, t0.z}, pb{t0.w, t1.x}, ez0{t1.y, t1.z}, ezc{t1.w, t2.x}, e10{t2.y, t2.z},
+                    e1c{t2.w, t3.x};
+                float tb;
+                split_coord(df_add(df_add(df_mul_f(rb, ca), pb), DF{-cb0, 0.0f}), jb, tb);
+                const DF E0 = df_add(ez0, df_mul_f(ezc, ca));  // centred height at v' = 0
+                const DF E1 = df_add(e10, df_mul_f(e1c, ca));
+                const float E = E1.hi, rE = __frcp_rn(E);
+                const float jf = rintf(fmaf(zc - E0.hi, rE, cv));  // anchor row: nearest the middle height
+                const DF ha = df_add(df_add(E0, df_mul_f(E1, jf - cv)), DF{-zc, 0.0f});
+                const float d1 = __fadd_rn(ha.hi, 1.0f) + ha.lo;
+                const float c0 = -d1 * rE;
+                // the row a height starts at: the very expression the lanes
+                // evaluate, monotone in z
+                auto row = [&](float z) { return __fadd_ru(__fmaf_rn(z, rE, c0), BT_MAGIC) - BT_MAGIC; };
+                const float r0 = -jf, rend = (float)a.nv - jf;  // the detector's rows, from the anchor
+                constexpr int ZS = ZT / NP;  // heights of a pair of the lanes
+#pragma unroll
+                for (int q = 0; q < NP; ++q) {
+                    const float rf = row((float)(-ZT / 2 + q * ZS)), rl = row((float)(-ZT / 2 + (q + 1) * ZS - 1));
+                    if (fabsf(rf) < 1.0e6f && fabsf(rl) < 1.0e6f && rf < rend && rl + 2.0f * rE + 2.0f > r0) on |= 1 << q;
+                }
+                if (!((t0.x != 0.0f) == (cls != 0) && jb >= -1 && jb < wb && !(jb < 0 && tb == 0.0f) && E > 0.0f &&
+                      fabsf(jf) < 1.0e6f && on))
+                    jb = -2;
+                rows = E > 0.501f && E < 1.0f ? (E > 0.667f ? 3 : 4) : (E > 0.401f ? 5 : 0);
+                te.E = E;
+                te.Elo = E1.lo;
+                te.d1 = d1;
+                te.rE = rE;
+                te.base = (long long)(SINO_PAD + ((size_t)i * a.nu + ju) * (a.nv + SINO_PAD)) +
+                          (long long)((int)jf - BT_MAGIC_BITS);
+                te.tb = tb;
+                te.rlo = BT_MAGIC + (r0 - (float)SINO_PAD);
+            }
+            auto sweep = [&](auto ltag) {
+                constexpr bool LOOP = decltype(ltag)::value;
+                const int key = (rows == 0) == LOOP ? jb : -2;
+                if (!__any_sync(FULL, key >= -1)) return;
+                // counting sort by jb
+                int run = 0, at = 0;
+#pragma unroll
+                for (int j = -1; j < W; ++j) {
+                    const unsigned g = __ballot_sync(FULL, key == j);
+                    if (key == j) at = run + __popc(g & ((1u << lane) - 1u));
+                    run += __popc(g);
+                }
+                if (key >= -1) tab[at] = te;
+                __syncwarp();
+                // bit masks over the table: entries of 3 rows, of 4, and of pair q
+                const unsigned bit = key >= -1 ? 1u << at : 0u;
+                unsigned m3 = __reduce_or_sync(FULL, rows == 3 ? bit : 0u), m4 = __reduce_or_sync(FULL, rows == 4 ? bit : 0u);
+                unsigned mq[NP];
+#pragma unroll
+                for (int q = 0; q < NP; ++q) mq[q] = __reduce_or_sync(FULL, (on >> q) & 1 ? bit : 0u);
+                float2 lo[NP], hi[NP];  // voxel columns j and j + 1
+#pragma unroll
+                for (int q = 0; q < NP; ++q) lo[q] = hi[q] = both(0.0f);
+                const ColEntry *t = tab;
+                float *dst = accw - NCH * ZP;
+#pragma unroll 1
+                for (int j = -1; j < W; ++j) {
+                    const int ng = __popc(__ballot_sync(FULL, key == j));
+#pragma unroll 1
+                    for (int e = 0; e < ng; ++e, ++t) {
+                        const ColEntry c = *t;
+                        const ST *anchor = sino + c.base;
+                        float2 p[NP];
+#pragma unroll
+                        for (int q = 0; q < NP; ++q) p[q] = both(0.0f);
+                        auto each = [&](auto f) {
+#pragma unroll
+                            for (int q = 0; q < NP; ++q)
+                                if (NP == 1 || (mq[q] & 1u)) p[q] = f(zl[q]);
+                        };
+                        if (LOOP) each([&](float2 z) { return bt_profile_loop<NCH>(c, anchor, a.nv, z); });
+                        else if (m3 & 1u) each([&](float2 z) { return bt_profile<3, NCH>(c, anchor, rspan, z); });
+                        else if (m4 & 1u) each([&](float2 z) { return bt_profile<4, NCH>(c, anchor, rspan, z); });
+                        else each([&](float2 z) { return bt_profile<5, NCH>(c, anchor, rspan, z); });
+                        m3 >>= 1;
+                        m4 >>= 1;
+#pragma unroll
+                        for (int q = 0; q < NP; ++q) mq[q] >>= 1;
+                        const float wl = 1.0f - c.tb;
+#pragma unroll
+                        for (int q = 0; q < NP; ++q) {
+                            lo[q] = fma_f2(both(wl), p[q], lo[q]);
+                            if (c.tb > 0.0f) hi[q] = fma_f2(both(c.tb), p[q], hi[q]);
+                        }
+                    }
+                    if (j >= 0) {
+#pragma unroll
+                        for (int q = 0; q < NP; ++q) {
+                            float *d = dst + q * (ZT / NP);
+                            d[0] += lo[q].x;
+                            d[NCH == 2 ? ZP : 32] += lo[q].y;
+                        }
+                    }
+                    dst += NCH * ZP;
+#pragma unroll
+                    for (int q = 0; q < NP; ++q) {
+                        lo[q] = hi[q];
+                        hi[q] = both(0.0f);
+                    }
+                }
+                __syncwarp();
+            };
+            sweep(std::false_type());
+            sweep(std::true_type());
+        }
+    }
+    // the block's BT_WARPS planes x W columns, the volume's rows in runs of W
+    // (class 1) or BT_WARPS (class 0) voxels
+    __syncthreads();
+    const size_t nvox = (size_t)a.n * a.n * a.n;
+    float *o = out + (size_t)part * NCH * nvox;
+    for (int t = tid; t < BT_WARPS * W * ZT; t += 32 * BT_WARPS) {
+        const int c = t % (BT_WARPS * W), zz = t / (BT_WARPS * W), z = z0 + zz;
+        const int w = cls ? c / W : c % BT_WARPS, j = cls ? c % W : c / BT_WARPS;
+        const int x = cls ? b0 + j : p0 + w, y = cls ? p0 + w : b0 + j;
+        if (x < a.n && y < a.n && z < a.n) {
+            const size_t idx = ((size_t)z * a.n + y) * a.n + x;
 #pragma unroll
             for (int q = 0; q < NCH; ++q) {
-                float v = acc[q][zz + 2][tid];
+                float v = acc[((w * W + j) * NCH + q) * ZP + zz];
                 if (accumulate) v += o[idx + q * nvox];
                 o[idx + q * nvox] = v;
             }
@@ -451,235 +678,10 @@ __global__ void __launch_bounds__(BS_THREADS)
     }
 }
 
-// Register form of the solver's A^T (separable geometry, weighted rows, one
-// channel) for grids whose detector rows are finer than the voxels along z:
-// 1/3 < E1 < 1 for every view, column and plane (LevelInfo::e1_lo / e1_hi).
-// As in the slab kernel a thread owns one (x, y) voxel column and ZS voxels
-// z0 .. z0 + ZS - 1 of it, but the slab lives in registers.  Measured from
-// z0 - 1, a detector column's row crossings rise by E1 < 1 per row, so the
-// unit interval j of heights, [j, j + 1), j = 0 .. ZS, holds floor(1/E1) or
-// ceil(1/E1) rows (K = ceil(1/E1) slots, the later ones predicated).  With
-// S_j the interval's sum of y and T_j its sum of y t (t = the row's height
-// above j), the tent weights give voxel z0 - 1 + j the share hb (S_j - T_j)
-// and voxel z0 + j the share hb T_j -- the slab kernel's two taps per row,
-// summed per interval, every accumulator index fixed at compile time.
-#ifndef MGCT_BR_BX
-#define MGCT_BR_BX 32
-#endif
-#ifndef MGCT_BR_WX
-#define MGCT_BR_WX 8
-#endif
-// a block is BR_TX x BR_TY voxel columns; a warp BR_WX x (32 / BR_WX) of them.
-// Measured per grid-0 launch at 256^3 / 720 views (512^3 / 1440): warps of
-// 32 x 1 columns 31.2 ms (452), 16 x 2 30.2 (442), 8 x 4 29.5 (435), and
-// 4 x 8 or 8 x 4 in 16 x 8 and 8 x 16 blocks 29.4-29.8 (433-439): on views
-// whose rays run along a warp's long side, its lanes' detector columns and
-// rows spread apart
-constexpr int BR_TX = MGCT_BR_BX, BR_TY = 128 / BR_TX, BR_THREADS = BR_TX * BR_TY;
-constexpr int BR_WX = MGCT_BR_WX, BR_WY = 32 / BR_WX;
-static_assert(BR_TX % BR_WX == 0 && BR_TY % BR_WY == 0, "warp tiles must tile the block");
-#ifndef MGCT_BR_Z
-#define MGCT_BR_Z 16
-#endif
-// measured at 256^3 / 720 views per grid-0 launch (slab kernel 42.5 ms):
-// 16 voxels, the later slots' rows loaded before their test, 40 registers
-// (12 blocks per SM), the exact column range 31.1 ms; with the cube bound's
-// column range 35.1 (each lane's weighted columns start at a different
-// iteration, so a warp runs more of the expensive ones); with 24 voxels
-// 37.9, with 8 voxels 57.1; with the loads behind the test 38.2; without the
-// register cap (118 registers) 55.7 (cube bound for these five)
-#ifndef MGCT_BR_UNCOND
-#define MGCT_BR_UNCOND 1
-#endif
-#ifndef MGCT_BR_MINB
-#define MGCT_BR_MINB 12
-#endif
-#ifndef MGCT_BR_EXACT
-#define MGCT_BR_EXACT 1
-#endif
-constexpr int BR_Z = MGCT_BR_Z;                        // voxels per thread along z
-constexpr float BR_E1_LO = 1.0f / 3.0f + 1e-3f;        // eligible grids: BR_E1_LO < E1 < BR_E1_HI
-constexpr float BR_E1_HI = 1.0f - 1e-3f;
-constexpr float BR_K2 = 0.5f + 1e-3f;                  // E1 above this: at most two rows per interval
-
-// One detector column's rows into acc: off is the element offset of the
-// first row (row v, height w in [0, E1) above z0 - 1) in the view's
-// sinogram.  EDGE: rows outside [0, nv) read as zero (not loaded).
-template <int ZS, int K, bool EDGE, typename ST>
-__device__ __forceinline__ void br_column(float (&acc)[ZS], const ST *__restrict__ sv, int off, int nu, float w,
-                                          float E1, float hb, int v, int nv) {
-#pragma unroll
-    for (int j = 0; j <= ZS; ++j) {
-        float y = 0.0f;
-        if (!EDGE || (unsigned)v < (unsigned)nv) y = to_f32(__ldg(sv + off));
-        float S = y, T = y * w;
-        float wn = w + E1;  // height of the next row above j
-        int adv = 1;
-#pragma unroll
-        for (int s = 1; s < K; ++s) {
-            if (MGCT_BR_UNCOND && !EDGE) {
-                // the row after the interval's last lies within the rows the
-                // launch checked, so the load need not wait for the test
-                const float yl = to_f32(__ldg(sv + off + s * nu));
-                const bool in = wn < 1.0f;
-                const float ys = in ? yl : 0.0f;
-                S += ys;
-                T = fmaf(ys, wn, T);
-                if (in) {
-                    wn += E1;
-                    adv = s + 1;
-                }
-            } else if (wn < 1.0f) {
-                float ys = 0.0f;
-                if (!EDGE || (unsigned)(v + s) < (unsigned)nv) ys = to_f32(__ldg(sv + off + s * nu));
-                S += ys;
-                T = fmaf(ys, wn, T);
-                wn += E1;
-                adv = s + 1;
-            }
-        }
-        if (j >= 1) acc[j - 1] = fmaf(hb, S - T, acc[j - 1]);
-        if (j < ZS) acc[j] = fmaf(hb, T, acc[j]);
-        w = wn - 1.0f;  // the first row of interval j + 1
-        off += adv * nu;
-        if (EDGE) v += adv;
-    }
-}
-
-// Detector column ju of the view whose sinogram is sv into acc, weighted hb:
-// E0 is the uncentred z crossing of its rays at v' = 0 and E1 its step per
-// row, at the voxel column's plane; the slab's intervals start at zlo.
-template <int ZS, typename ST>
-__device__ __forceinline__ void br_add_column(float (&acc)[ZS], const ST *__restrict__ sv, int ju, int nu, int nv,
-                                              float E0, float E1, float hb, float zlo, float cv) {
-    // the launch checks the grid's range of E1; this keeps every read in
-    // bounds whatever the table holds
-    if (!(E1 > 0.3f && E1 < 1.0f)) return;
-    const float rE = __frcp_rn(E1);
-    // first row at or above z0 - 1 (one correction for the rounded quotient)
-    float vf = ceilf(fmaf(zlo - E0, rE, cv));
-    if (!(fabsf(vf) < 1.0e7f)) return;
-    float w = fmaf(vf - cv, E1, E0) - zlo;
-    if (w < 0.0f) {
-        vf += 1.0f;
-        w += E1;
-    } else if (w >= E1) {
-        vf -= 1.0f;
-        w -= E1;
-    }
-    const int vs = (int)vf;
-    // rows read: those of heights [0, ZS + 1), at most (ZS + 1) / E1 + 1 (the
-    // truncation below loses one), one more for the drift of the stepped
-    // heights, two after the last that the unconditional slots may read, and
-    // one spare
-    constexpr int nrb_max = (int)((float)(ZS + 1) / BR_E1_LO) + 6;
-    const int nrb = min(nrb_max, (int)((float)(ZS + 1) * rE) + 6);
-    if (vs >= nv || vs + nrb <= 0) return;
-    const int off = vs * nu + ju;
-    if (vs >= 0 && vs + nrb <= nv) {
-        if (E1 > BR_K2) br_column<ZS, 2, false>(acc, sv, off, nu, w, E1, hb, vs, nv);
-        else br_column<ZS, 3, false>(acc, sv, off, nu, w, E1, hb, vs, nv);
-    } else {
-        if (E1 > BR_K2) br_column<ZS, 2, true>(acc, sv, off, nu, w, E1, hb, vs, nv);
-        else br_column<ZS, 3, true>(acc, sv, off, nu, w, E1, hb, vs, nv);
-    }
-}
-
-template <typename ST, int ZS>
-__global__ void __launch_bounds__(BR_THREADS, MGCT_BR_MINB)
-    k_backproject_reg(BPArgs a, const float4 *__restrict__ cols, const ST *__restrict__ sino,
-                      float *__restrict__ out, int accumulate) {
-    const int tid = threadIdx.x;
-    const int w = tid >> 5, l = tid & 31;
-    const int jx = blockIdx.x * BR_TX + (w % (BR_TX / BR_WX)) * BR_WX + l % BR_WX;
-    const int jy = blockIdx.y * BR_TY + (w / (BR_TX / BR_WX)) * BR_WY + l / BR_WX;
-    // blockIdx.z = split * (z-slabs) + slab, as in k_backproject_slab
-    const int zblocks = gridDim.z / a.splits;
-    const int split = blockIdx.z / zblocks;
-    const int z0 = (blockIdx.z - split * zblocks) * ZS;
-    const int per = (a.nviews + a.splits - 1) / a.splits;
-    const int i0 = split * per, i1 = min(a.nviews, i0 + per);
-    if (jx >= a.n || jy >= a.n) return;
-    float acc[ZS];
-#pragma unroll
-    for (int q = 0; q < ZS; ++q) acc[q] = 0.0f;
-    const float ic = 0.5f * (float)(a.n - 1);
-    const float cu = 0.5f * (float)(a.nu - 1), cv = 0.5f * (float)(a.nv - 1);
-    const float cx = (float)jx - ic, cy = (float)jy - ic;
-    const float zlo = (float)z0 - 1.0f;  // interval 0 starts here
-    const size_t view_elems = (size_t)a.nu * a.nv;
-    for (int i = i0; i < i1; ++i) {
-        const int k = a.view0 + i * a.stride;
-        const float *G = reinterpret_cast<const float *>(a.views + k);
-        const float X = (float)jx - __ldg(G + 0), Y = (float)jy - __ldg(G + 1);
-        const float Q0 = __ldg(G + 12), Q1 = __ldg(G + 13), Q6 = __ldg(G + 18), Q7 = __ldg(G + 19);
-        const float q0 = fmaf(Q1, Y, Q0 * X), q2 = fmaf(Q7, Y, Q6 * X);
-        int ulo, uhi;
-        if (MGCT_BR_EXACT) {
-            // a column of x-major rays weights this voxel column iff its rays
-            // cross the plane x = jx strictly between y = jy - 1 and jy + 1,
-            // i.e. iff its u lies between the projections of those two
-            // points; likewise (jx -+ 1, jy) for y-major rays.  Both intervals
-            // hold the voxel column's own projection, so their union is the
-            // interval from the least to the greatest of the four.
-            const float ua = (q0 - Q1) * __frcp_rn(q2 - Q7), ub = (q0 + Q1) * __frcp_rn(q2 + Q7);
-            const float uc = (q0 - Q0) * __frcp_rn(q2 - Q6), ud = (q0 + Q0) * __frcp_rn(q2 + Q6);
-            const float umin = fminf(fminf(ua, ub), fminf(uc, ud)), umax = fmaxf(fmaxf(ua, ub), fmaxf(uc, ud));
-            ulo = max(0, (int)ceilf(umin + cu - 1e-3f));
-            uhi = min(a.nu - 1, (int)floorf(umax + cu + 1e-3f));
-        } else {
-            // projected u range of the voxel column (the cube bound)
-            const float u0 = q0 * __frcp_rn(q2);
-            const float hu = (fabsf(Q0 - u0 * Q6) + fabsf(Q1 - u0 * Q7)) * __frcp_rn(q2 - __ldg(G + 21));
-            ulo = max(0, (int)ceilf(u0 - hu + cu - 1e-3f));
-            uhi = min(a.nu - 1, (int)floorf(u0 + hu + cu + 1e-3f));
-        }
-        const ST *__restrict__ sv = sino + (size_t)i * view_elems;
-        const float4 *__restrict__ ct = cols + (size_t)k * a.nu * 2;
-        for (int ju = ulo; ju <= uhi; ++ju) {
-            const float4 t0 = __ldg(ct + 2 * ju);
-            const float4 t1 = __ldg(ct + 2 * ju + 1);
-            const bool ay = t0.x != 0.0f;
-            const float ca = ay ? cy : cx, cb = ay ? cx : cy;
-            const float hb = 1.0f - fabsf(fmaf(ca, t0.y, t0.z) - cb);
-            if (hb <= 0.0f) continue;
-            br_add_column<ZS>(acc, sv, ju, a.nu, a.nv, fmaf(ca, t1.x, t0.w) + ic, fmaf(ca, t1.z, t1.y), hb, zlo, cv);
-        }
-    }
-    const size_t nvox = (size_t)a.n * a.n * a.n;
-    float *o = out + (size_t)split * nvox;
-#pragma unroll
-    for (int zz = 0; zz < ZS; ++zz) {
-        const int z = z0 + zz;
-        if (z < a.n) {
-            const size_t idx = ((size_t)z * a.n + jy) * a.n + jx;
-            float v = acc[zz];
-            if (accumulate) v += o[idx];
-            o[idx] = v;
-        }
-    }
-}
-
-// Column table (see LevelInfo::d_cols): one thread per (view, column); the
-// axis choice is the projector's own ray_dir() at v' = 0.
-__global__ void k_column_table(const ViewGeom *__restrict__ views, int K, int nu, float4 *__restrict__ cols) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= K * nu) return;
-    const int k = t / nu, ju = t % nu;
-    const ViewGeom &G = views[k];
-    const float up = (float)ju - 0.5f * (float)(nu - 1);
-    const RayDir d = ray_dir(G, up, 0.0f);
-    const float wa = d.ax ? d.wy : d.wx, wb = d.ax ? d.wx : d.wy;
-    const float rinv = __frcp_rn(wa);
-    const float *N = d.ax ? G.NY : G.NX;
-    cols[2 * (size_t)t] = make_float4(d.ax ? 1.0f : 0.0f, wb * rinv, fmaf(up, N[1], N[0]) * rinv,
-                                      fmaf(up, N[4], N[3]) * rinv);
-    cols[2 * (size_t)t + 1] = make_float4(G.Wc[2] * rinv, N[5] * rinv, G.Ev[2] * rinv, 0.0f);
-}
-
-// Double-float column table (see LevelInfo::d_cols_df): same axis choice as
-// k_column_table; the quotients by w_a are taken in double-float from the
-// view table's double-float fields.
+// Double-float column table (see LevelInfo::d_cols_df), one thread per (view,
+// column): the axis choice is the projector's own ray_dir() at v' = 0; the
+// quotients by w_a are taken in double-float from the view table's
+// double-float fields.
 __global__ void k_column_table_df(const ViewGeom *__restrict__ views, int K, int nu, float4 *__restrict__ cols) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= K * nu) return;
@@ -699,11 +701,30 @@ __global__ void k_column_table_df(const ViewGeom *__restrict__ views, int K, int
     const DF ezc = df_mul(df_affine(G.Wc[2], G.Wc_lo[2], G.Eu[2], G.Eu_lo[2], G.Ev[2], G.Ev_lo[2], up, 0.0f), rinv);
     const DF e10 = df_mul(DF{N[5], Nl[5]}, rinv);
     const DF e1c = df_mul(DF{G.Ev[2], G.Ev_lo[2]}, rinv);
-    float4 *o = cols + 4 * (size_t)t;
+    float4 *o = cols + (size_t)k * 4 * nu + ju;
     o[0] = make_float4(d.ax ? 1.0f : 0.0f, rb.hi, rb.lo, pb.hi);
-    o[1] = make_float4(pb.lo, ez0.hi, ez0.lo, ezc.hi);
-    o[2] = make_float4(ezc.lo, e10.hi, e10.lo, e1c.hi);
-    o[3] = make_float4(e1c.lo, 0.0f, 0.0f, 0.0f);
+    o[(size_t)nu] = make_float4(pb.lo, ez0.hi, ez0.lo, ezc.hi);
+    o[2 * (size_t)nu] = make_float4(ezc.lo, e10.hi, e10.lo, e1c.hi);
+    o[3 * (size_t)nu] = make_float4(e1c.lo, 0.0f, 0.0f, 0.0f);
+}
+
+// First and last detector column of each ray class per view (LevelInfo::
+// d_ranges; an empty class has first > last), a warp per view.
+__global__ void k_class_ranges(const float4 *__restrict__ cols, int K, int nu, int2 *__restrict__ ranges) {
+    const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (k >= K) return;
+    int lo[2] = {nu, nu}, hi[2] = {-1, -1};
+    for (int u = lane; u < nu; u += 32) {
+        const int c = __ldg(cols + (size_t)k * 4 * nu + u).x != 0.0f;
+        lo[c] = min(lo[c], u);
+        hi[c] = max(hi[c], u);
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        lo[c] = __reduce_min_sync(0xffffffffu, lo[c]);
+        hi[c] = __reduce_max_sync(0xffffffffu, hi[c]);
+        if (lane == 0) ranges[2 * k + c] = make_int2(lo[c], hi[c]);
+    }
 }
 
 // out = (accumulate ? out : 0) + sum over s of part[s], in order of s.
@@ -716,58 +737,92 @@ __global__ void k_sum_splits(size_t len, int splits, const float *__restrict__ p
     }
 }
 
-// Number of view ranges for a slab launch of `blocks` blocks: enough for
-// about four waves of resident blocks in all, as grid 0 has (coarse grids and
-// OS-EMTR subsets otherwise fill a fraction of the SMs, and a launch of one
-// or two waves loses its tail), at most 16 and what `cap` floats of partial
-// volumes hold.
-template <typename KF>
-int slab_splits(KF kernel, int blocks, int nviews, size_t vol_floats, size_t cap) {
-    int dev = 0, sms = 0, occ = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
-                                                  cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, BS_THREADS, 0) != cudaSuccess) {
-        cudaGetLastError();
-        return 1;
+// out = (accumulate ? out : 0) + the sum of `parts` partial volumes, as a
+// balanced tree over their (zero-extended) 32: the partial sums of a float32
+// chain of up to 32 would cost more digits than the back-projection itself.
+template <int P>
+__device__ __forceinline__ float tree_sum(const float *__restrict__ part, size_t len, int first, int parts) {
+    if (first >= parts) return 0.0f;
+    if constexpr (P == 1) return __ldg(part + (size_t)first * len);
+    else return tree_sum<P / 2>(part, len, first, parts) + tree_sum<P / 2>(part, len, first + P / 2, parts);
+}
+__global__ void k_sum_parts(size_t len, int parts, const float *__restrict__ part, float *__restrict__ out,
+                            int accumulate) {
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (size_t)gridDim.x * blockDim.x) {
+        const float v = tree_sum<32>(part + i, len, 0, parts);
+        out[i] = accumulate ? out[i] + v : v;
     }
-    int sp = (4 * sms * occ + blocks - 1) / blocks;
-    if (sp > 16) sp = 16;
-    if (sp > nviews) sp = nviews;
-    if ((size_t)sp * vol_floats > cap) sp = (int)(cap / vol_floats);
-    return sp < 1 ? 1 : sp;
 }
 
-// The register kernel's launch (see k_backproject_reg), with the slab
-// kernel's view splits.
-template <typename ST>
-int launch_backproject_reg(const LevelInfo &L, BPArgs a, const ST *sino, float *out, int accumulate, cudaStream_t s,
-                           float *split_buf, size_t cap) {
-    dim3 grid((L.n + BR_TX - 1) / BR_TX, (L.n + BR_TY - 1) / BR_TY, (L.n + BR_Z - 1) / BR_Z);
-    const size_t vol_floats = (size_t)L.n * L.n * L.n;
-    if (split_buf && a.nviews > 1)
-        a.splits = slab_splits(k_backproject_reg<ST, BR_Z>, (int)(grid.x * grid.y * grid.z), a.nviews, vol_floats,
-                               cap);
-    if (a.splits == 1) {
-        MGCT_KERNEL(KK_BACKPROJECT, s,
-                    k_backproject_reg<ST, BR_Z><<<grid, BR_THREADS, 0, s>>>(a, L.d_cols, sino, out, accumulate));
-    } else {
-        grid.z *= a.splits;
-        MGCT_KERNEL(KK_BACKPROJECT, s,
-                    k_backproject_reg<ST, BR_Z><<<grid, BR_THREADS, 0, s>>>(a, L.d_cols, sino, split_buf, 0));
-        const int sb = (int)((vol_floats + 255) / 256 < 4096 ? (vol_floats + 255) / 256 : 4096);
-        MGCT_KERNEL(KK_BACKPROJECT, s, k_sum_splits<<<sb, 256, 0, s>>>(vol_floats, a.splits, split_buf, out, accumulate));
+}  // namespace mgct
+
+#include "backproject16.cuh"
+
+namespace mgct {
+
+// Number of view ranges for a plane-kernel launch of `blocks` tiles: the one
+// that fills whole waves of resident blocks best (a launch of 3.4 waves takes
+// as long as one of 4; coarse grids and OS-EMTR subsets fill a fraction of
+// one), at most 16 and `most`.  Each range beyond the first has to gain 4 %
+// for its partial volume and set-up.
+inline int plane_splits(int resident, int blocks, int nviews, int most) {
+    int best = 1;
+    double cost = 1e300;
+    for (int sp = 1; sp <= 16 && sp <= nviews && (sp == 1 || sp <= most); ++sp) {
+        const double waves = (double)(((long long)blocks * sp + resident - 1) / resident);
+        const double c = waves / sp * (1.0 + 0.04 * (sp - 1));
+        if (c < cost) {
+            cost = c;
+            best = sp;
+        }
     }
+    return best;
+}
+
+template <int NCH, int NP, typename ST>
+int launch_backproject_plane(const LevelInfo &L, BPArgs a, const ST *sino, float *out, int accumulate, cudaStream_t s,
+                             float *split_buf, size_t cap) {
+    using T = PlaneTile<NCH, NP>;
+    auto *kernel = k_backproject_plane<NCH, NP, ST>;
+    constexpr size_t smem = T::smem;
+    static_assert(smem <= 48 * 1024, "within the default shared-memory limit");
+    dim3 grid((L.n + T::W - 1) / T::W, (L.n + BT_WARPS - 1) / BT_WARPS, (L.n + T::ZT - 1) / T::ZT);
+    const size_t vol_floats = (size_t)NCH * L.n * L.n * L.n;
+    const int room = split_buf ? (int)(cap / vol_floats < 64 ? cap / vol_floats : 64) : 0;
+    if (room < 2) {
+        // no room for partial volumes: the two ray classes one after the other
+        for (a.cls = 1; a.cls >= 0; --a.cls)
+            MGCT_KERNEL(KK_BACKPROJECT, s,
+                        kernel<<<grid, 32 * BT_WARPS, smem, s>>>(a, L.d_cols_df, L.d_ranges, sino, out, accumulate || a.cls == 0));
+        return MGCT_OK;
+    }
+    int dev = 0, sms = 0, occ = 0;
+    MGCT_TRY(check_cuda(cudaGetDevice(&dev), "device"));
+    MGCT_TRY(check_cuda(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device"));
+    MGCT_TRY(check_cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, 32 * BT_WARPS, smem), "occupancy"));
+    a.splits = plane_splits(sms * (occ > 0 ? occ : 1), 2 * (int)(grid.x * grid.y * grid.z), a.nviews, room / 2);
+    const int parts = 2 * a.splits;
+    grid.z *= parts;
+    MGCT_KERNEL(KK_BACKPROJECT, s, kernel<<<grid, 32 * BT_WARPS, smem, s>>>(a, L.d_cols_df, L.d_ranges, sino, split_buf, 0));
+    const int sb = (int)((vol_floats + 255) / 256 < 4096 ? (vol_floats + 255) / 256 : 4096);
+    MGCT_KERNEL(KK_BACKPROJECT, s, k_sum_parts<<<sb, 256, 0, s>>>(vol_floats, parts, split_buf, out, accumulate));
     return MGCT_OK;
 }
 
-// NCH = 2 writes channel c to out + c * n^3.  WEIGHTED: the sinogram carries
-// each ray's dl already (internal solver path).  split_buf (cap floats, or
-// NULL): scratch for partial volumes, with which an under-filled slab launch
-// splits its views into ranges summed afterwards in a fixed order.
-template <int NCH, typename ST, bool WEIGHTED = false>
-int launch_backproject(const mgct_geom *g, int level, int view0, int nviews, int stride, const ST *sino,
-                       float *out, int accumulate, cudaStream_t s, float *split_buf = nullptr, size_t cap = 0) {
-    const LevelInfo &L = g->lev[level];
+// A^T of a weighted sinogram stored [view][u][v] on a separable geometry.
+// Two pairs a lane halve the per-column work of a height, one wastes less of
+// the last tile: one where the tiles of the larger kind hold over a quarter
+// more heights.
+template <int NCH, typename ST>
+int launch_backproject_cols(const LevelInfo &L, const BPArgs &a, const ST *sino, float *out, int accumulate,
+                            cudaStream_t s, float *split_buf, size_t cap) {
+    constexpr int Z1 = PlaneTile<NCH, 1>::ZT, Z2 = PlaneTile<NCH, 2>::ZT;
+    const int t1 = (L.n + Z1 - 1) / Z1 * Z1, t2 = (L.n + Z2 - 1) / Z2 * Z2;
+    if (4 * t2 <= 5 * t1) return launch_backproject_plane<NCH, 2, ST>(L, a, sino, out, accumulate, s, split_buf, cap);
+    return launch_backproject_plane<NCH, 1, ST>(L, a, sino, out, accumulate, s, split_buf, cap);
+}
+
+inline BPArgs bp_args(const LevelInfo &L, int view0, int nviews, int stride) {
     BPArgs a;
     a.views = L.d_views;
     a.n = L.n;
@@ -778,62 +833,75 @@ int launch_backproject(const mgct_geom *g, int level, int view0, int nviews, int
     a.stride = stride;
     a.nviews = nviews;
     a.splits = 1;
-    if (MGCT_BS_REG && NCH == 1 && g->separable && WEIGHTED && L.d_cols && L.e1_lo > BR_E1_LO &&
-        L.e1_hi < BR_E1_HI && (size_t)L.nu * (L.nv + 64) < ((size_t)1 << 31)) {
-        if constexpr (NCH == 1) return launch_backproject_reg<ST>(L, a, sino, out, accumulate, s, split_buf, cap);
-    } else if (g->separable && WEIGHTED && L.d_cols) {
-        constexpr int Z = SlabCfg<NCH>::Z;
-        dim3 grid((L.n + BS_TX - 1) / BS_TX, (L.n + BS_TY - 1) / BS_TY, (L.n + Z - 1) / Z);
-        const size_t vol_floats = (size_t)NCH * L.n * L.n * L.n;
-        if (split_buf && nviews > 1)
-            a.splits = slab_splits(k_backproject_slab<NCH, ST>, (int)(grid.x * grid.y * grid.z), nviews, vol_floats,
-                                   cap);
-        if (a.splits == 1) {
-            MGCT_KERNEL(KK_BACKPROJECT, s,
-                        k_backproject_slab<NCH, ST><<<grid, BS_THREADS, 0, s>>>(a, L.d_cols, sino, out, accumulate));
-        } else {
-            grid.z *= a.splits;
-            MGCT_KERNEL(KK_BACKPROJECT, s,
-                        k_backproject_slab<NCH, ST><<<grid, BS_THREADS, 0, s>>>(a, L.d_cols, sino, split_buf, 0));
-            const int sb = (int)((vol_floats + 255) / 256 < 4096 ? (vol_floats + 255) / 256 : 4096);
-            MGCT_KERNEL(KK_BACKPROJECT, s,
-                        k_sum_splits<<<sb, 256, 0, s>>>(vol_floats, a.splits, split_buf, out, accumulate));
-        }
-    } else if (g->separable) {
-        const int zper = BP_BZ * BPS_ZB;
-        dim3 grid((L.n + BP_BX - 1) / BP_BX, (L.n + BP_BY - 1) / BP_BY, (L.n + zper - 1) / zper);
-        MGCT_KERNEL(KK_BACKPROJECT, s,
-                    k_backproject_sep<NCH, ST, WEIGHTED><<<grid, dim3(BP_BX, BP_BY, BP_BZ), 0, s>>>(a, L.d_cols_df, sino, out, accumulate));
-    } else {
-        dim3 grid((L.n + BP_BX - 1) / BP_BX, (L.n + BP_BY - 1) / BP_BY, (L.n + BP_BZ - 1) / BP_BZ);
-        MGCT_KERNEL(KK_BACKPROJECT, s,
-                    k_backproject<NCH, ST, WEIGHTED><<<grid, dim3(BP_BX, BP_BY, BP_BZ), 0, s>>>(a, sino, out, accumulate));
+    a.cls = -1;
+    return a;
+}
+
+// NCH = 2 writes channel c to out + c * n^3.  WEIGHTED: the sinogram carries
+// each ray's dl already (internal solver path) and is stored as
+// weighted_strides says.  split_buf (cap floats, or NULL):
+// scratch for partial volumes.
+template <int NCH, typename ST, bool WEIGHTED = false>
+int launch_backproject(const mgct_geom *g, int level, int view0, int nviews, int stride, const ST *sino,
+                       float *out, int accumulate, cudaStream_t s, float *split_buf = nullptr, size_t cap = 0) {
+    const LevelInfo &L = g->lev[level];
+    const BPArgs a = bp_args(L, view0, nviews, stride);
+    if (g->separable && WEIGHTED) {
+        if constexpr (sizeof(ST) == 2) return launch_backproject16<ST>(L, a, sino, out, accumulate, s, split_buf, cap);
+        else return launch_backproject_cols<NCH, ST>(L, a, sino, out, accumulate, s, split_buf, cap);
     }
+    if constexpr (!WEIGHTED) {
+        if (g->separable) {
+            const int zper = BP_BZ * BPS_ZB;
+            dim3 grid((L.n + BP_BX - 1) / BP_BX, (L.n + BP_BY - 1) / BP_BY, (L.n + zper - 1) / zper);
+            MGCT_KERNEL(KK_BACKPROJECT, s,
+                        k_backproject_sep<NCH, ST, WEIGHTED><<<grid, dim3(BP_BX, BP_BY, BP_BZ), 0, s>>>(a, L.d_cols_df, sino, out, accumulate));
+            return MGCT_OK;
+        }
+    }
+    dim3 grid((L.n + BP_BX - 1) / BP_BX, (L.n + BP_BY - 1) / BP_BY, (L.n + BP_BZ - 1) / BP_BZ);
+    MGCT_KERNEL(KK_BACKPROJECT, s,
+                k_backproject<NCH, ST, WEIGHTED><<<grid, dim3(BP_BX, BP_BY, BP_BZ), 0, s>>>(a, sino, out, accumulate));
     return MGCT_OK;
 }
 
 // The public A^T on tilt-free geometries.  Each ray's path length per plane,
 // dl = h sqrt(1 + rb^2 + rz^2) (the projector's weight; rb per column, rz
 // linear in v', both from the double-float column table), is applied to the
-// caller's sinogram in one pass over it, written to the handle's quad scratch,
-// and the weighted rows are splatted by the double-float-anchored slab
-// kernel: the solver's scatter, for one extra read and write of the sinogram.
+// caller's sinogram in one pass over it, which also turns it to [view][u][v]
+// with its zero rows (32 x 32 tiles through shared memory), into the handle's
+// quad scratch; the
+// plane kernel then takes it like the solver's residual.
 template <typename ST>
-__global__ void k_weight_rays(BPArgs a, const float4 *__restrict__ cols, const ST *__restrict__ sino,
-                              float *__restrict__ w) {
-    const int ju = blockIdx.x * blockDim.x + threadIdx.x;
-    if (ju >= a.nu) return;
-    const int jv = blockIdx.y, i = blockIdx.z;
+__global__ void __launch_bounds__(256)
+    k_weight_rays(BPArgs a, const float4 *__restrict__ cols, const ST *__restrict__ sino, float *__restrict__ w) {
+    __shared__ float tile[32][33];
+    const int u0 = blockIdx.x * 32, v0 = blockIdx.y * 32, i = blockIdx.z;
     const int k = a.view0 + i * a.stride;
-    const float *c = reinterpret_cast<const float *>(cols + ((size_t)k * a.nu + ju) * 4);
-    const float rb = __ldg(c + 1), ezc = __ldg(c + 7), e1c = __ldg(c + 11);  // rb, (Wc_z + u' Eu_z)/w_a, Ev_z/w_a
-    const float rz = fmaf((float)jv - 0.5f * (float)(a.nv - 1), e1c, ezc);
-    const float dl = sqrtf(fmaf(rz, rz, fmaf(rb, rb, 1.0f))) * a.h;
-    const size_t idx = ((size_t)i * a.nv + jv) * a.nu + ju;
-    w[idx] = dl * to_f32(__ldg(sino + idx));
+    const float4 *c = cols + (size_t)k * 4 * a.nu;
+    const size_t base = (size_t)i * a.nv * a.nu;
+    const int pitch = a.nv + SINO_PAD;
+    const int ju = u0 + threadIdx.x;
+    if (blockIdx.x + blockIdx.y + blockIdx.z == 0 && threadIdx.y == 0 && threadIdx.x < SINO_PAD) w[threadIdx.x] = 0.0f;
+    if (ju < a.nu) {
+        // rb, (Wc_z + u' Eu_z) / w_a, Ev_z / w_a
+        const float rb = __ldg(c + ju).y, ezc = __ldg(c + a.nu + ju).w, e1c = __ldg(c + 2 * a.nu + ju).w;
+        for (int r = threadIdx.y; r < 32; r += 8) {
+            tile[r][threadIdx.x] = 0.0f;  // the zero rows
+            if (v0 + r >= a.nv) continue;
+            const float rz = fmaf((float)(v0 + r) - 0.5f * (float)(a.nv - 1), e1c, ezc);
+            const float dl = sqrtf(fmaf(rz, rz, fmaf(rb, rb, 1.0f))) * a.h;
+            tile[r][threadIdx.x] = dl * to_f32(__ldg(sino + base + (size_t)(v0 + r) * a.nu + ju));
+        }
+    }
+    __syncthreads();
+    const int jv = v0 + threadIdx.x;
+    if (jv < pitch)
+        for (int r = threadIdx.y; r < 32 && u0 + r < a.nu; r += 8)
+            w[SINO_PAD + ((size_t)i * a.nu + u0 + r) * pitch + jv] = tile[threadIdx.x][r];
 }
 
-// Runs the public A^T through k_weight_rays and the slab kernel, in chunks of
+// Runs the public A^T through k_weight_rays and the plane kernel, in chunks of
 // views that fit the quad scratch, and sets *ran; leaves *ran = 0 (nothing
 // launched) where it does not apply: tilted detectors, no views, or a
 // scratch smaller than one view.
@@ -844,31 +912,22 @@ int launch_backproject_public(const mgct_geom *g, int level, int view0, int nvie
     const LevelInfo &L = g->lev[level];
     const size_t view_elems = (size_t)L.nu * L.nv;
     const size_t cap = 2 * quad_elems(g->lev[0].n) * 4;  // floats in the quad scratch
-    if (!g->separable || !L.d_cols_df || nviews < 1 || cap < view_elems || L.nv > 65535) return MGCT_OK;
-    size_t chunk = cap / view_elems;
+    const size_t padded = (size_t)L.nu * (L.nv + SINO_PAD);  // a view of weighted rays
+    if (!g->separable || !L.d_cols_df || nviews < 1 || cap < padded + SINO_PAD || L.nv > 65535) return MGCT_OK;
+    size_t chunk = (cap - SINO_PAD) / padded;
     if (chunk > (size_t)nviews) chunk = nviews;
     if (chunk > 65535) chunk = 65535;
     float *w = static_cast<float *>(g->d_scratch_quads);
-    BPArgs a;
-    a.views = L.d_views;
-    a.n = L.n;
-    a.nu = L.nu;
-    a.nv = L.nv;
-    a.h = (float)L.h;
-    a.stride = stride;
-    a.splits = 1;
-    constexpr int Z = SlabCfg<1>::Z;
-    const dim3 grid((L.n + BS_TX - 1) / BS_TX, (L.n + BS_TY - 1) / BS_TY, (L.n + Z - 1) / Z);
     for (int c0 = 0; c0 < nviews; c0 += (int)chunk) {
         const int cn = nviews - c0 < (int)chunk ? nviews - c0 : (int)chunk;
-        a.view0 = view0 + c0 * stride;
-        a.nviews = cn;
-        const dim3 wgrid((L.nu + 127) / 128, L.nv, cn);
+        const BPArgs a = bp_args(L, view0 + c0 * stride, cn, stride);
+        const dim3 wgrid((L.nu + 31) / 32, (L.nv + SINO_PAD + 31) / 32, cn);
         MGCT_KERNEL(KK_BACKPROJECT, s,
-                    k_weight_rays<ST><<<wgrid, 128, 0, s>>>(a, L.d_cols_df, sino + (size_t)c0 * view_elems, w));
-        MGCT_KERNEL(KK_BACKPROJECT, s,
-                    k_backproject_slab<1, float, true><<<grid, BS_THREADS, 0, s>>>(a, L.d_cols_df, w, out,
-                                                                                    (accumulate || c0) ? 1 : 0));
+                    k_weight_rays<ST><<<wgrid, dim3(32, 8), 0, s>>>(a, L.d_cols_df, sino + (size_t)c0 * view_elems, w));
+        // what the weighted rays leave of the scratch holds partial volumes
+        const size_t used = ((size_t)cn * padded + SINO_PAD + 63) & ~(size_t)63;
+        MGCT_TRY((launch_backproject_cols<1, float>(L, a, w, out, (accumulate || c0) ? 1 : 0, s, w + used,
+                                                    cap > used ? cap - used : 0)));
     }
     *ran = 1;
     return MGCT_OK;

@@ -60,11 +60,12 @@ struct LevelInfo {
     int n, nu, nv;
     double h, pitch;
     ViewGeom *d_views;  // device [K]
-    float4 *d_cols;     // device [K][nu][2] detector-column table (separable geometries), or NULL
-    float4 *d_cols_df;  // device [K][nu][4] the same quantities in double-float, or NULL
-    // range of the column table's z step per detector row, E1 = e10 + c_a e1c,
-    // over every view, column and voxel-centre plane c_a (separable geometries)
+    float4 *d_cols_df;  // device [K][4][nu] detector-column table in double-float (separable geometries), or NULL
+    float4 *d_cols;     // device [K][nu][2] the same in float32 (16-bit storage's back-projector), or NULL
+    // range of that table's z step per detector row, E1 = e10 + c_a e1c, over
+    // every view, column and voxel-centre plane c_a
     float e1_lo, e1_hi;
+    int2 *d_ranges;     // device [K][2] first and last column of x-major and of y-major rays (with d_cols_df)
 };
 
 // Detector-column table of a separable geometry (no detector tilt): for view
@@ -73,13 +74,12 @@ struct LevelInfo {
 // centred voxel coordinates along the column's major axis and the other
 // horizontal axis, the back-projector needs
 //   e_b = c_a rb + pb - c_b,   E0 + c_z = ez0 + c_a ezc,   E1 = e10 + c_a e1c.
-// Entry: {ax, rb, pb, ez0}, {ezc, e10, e1c, 0}.
-int launch_column_table(const mgct_geom *g, int level, cudaStream_t s);
-// The same column quantities as double-float pairs (hi, lo), for the public
-// back-projector's accuracy at large N: entry {ax, rb, rb_lo, pb},
-// {pb_lo, ez0, ez0_lo, ezc}, {ezc_lo, e10, e10_lo, e1c}, {e1c_lo, 0, 0, 0}
-// (centred: E0 + c_z = ez0 + c_a ezc).
+// as double-float pairs (hi, lo), in four float4 per column, {ax, rb, rb_lo,
+// pb}, {pb_lo, ez0, ez0_lo, ezc}, {ezc_lo, e10, e10_lo, e1c}, {e1c_lo, 0, 0,
+// 0} (centred: E0 + c_z = ez0 + c_a ezc), each an array over the columns.
 int launch_column_table_df(const mgct_geom *g, int level, cudaStream_t s);
+// In float32: entry {ax, rb, pb, ez0}, {ezc, e10, e1c, 0}.
+int launch_column_table(const mgct_geom *g, int level, cudaStream_t s);
 
 }  // namespace mgct
 
@@ -267,6 +267,15 @@ inline size_t project_blocks_any(int nu, int nv, int nviews) {
     const size_t a = project_blocks(nu, nv, nviews), b = project_blocks_col(nu, nv, nviews);
     return a > b ? a : b;
 }
+
+// ---------------------------------------------------------------------------
+// Weighted sinograms of separable geometries: zero rows before every detector
+// column and after the last, as many as the back-projector's profile reads.
+// ---------------------------------------------------------------------------
+constexpr int SINO_PAD = 5;
+inline size_t padded_sino_elems(size_t views, int nu, int nv) { return views * nu * (nv + SINO_PAD) + SINO_PAD; }
+// clears those rows of `columns` columns of nv rows, `elem` bytes an element
+int launch_zero_pads(size_t columns, int nv, int elem, void *sino, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Internal kernels used across translation units (host launchers)

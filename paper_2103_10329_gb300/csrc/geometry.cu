@@ -255,6 +255,8 @@ static int upload_tables(mgct_geom *g) {
         if (!L.d_cols_df)
             MGCT_TRY(check_cuda(cudaMalloc(&L.d_cols_df, (size_t)K * L.nu * 4 * sizeof(float4)),
                                 "allocate column table"));
+        if (!L.d_ranges)
+            MGCT_TRY(check_cuda(cudaMalloc(&L.d_ranges, (size_t)K * 2 * sizeof(int2)), "allocate column ranges"));
         MGCT_TRY(launch_column_table(g, l, 0));
         MGCT_TRY(launch_column_table_df(g, l, 0));
     }
@@ -297,6 +299,7 @@ void mgct_geometry_destroy(mgct_geom *g) {
         if (g->lev[l].d_views) cudaFree(g->lev[l].d_views);
         if (g->lev[l].d_cols) cudaFree(g->lev[l].d_cols);
         if (g->lev[l].d_cols_df) cudaFree(g->lev[l].d_cols_df);
+        if (g->lev[l].d_ranges) cudaFree(g->lev[l].d_ranges);
     }
     if (g->d_scratch_vol) cudaFree(g->d_scratch_vol);
     if (g->d_scratch_quads) cudaFree(g->d_scratch_quads);

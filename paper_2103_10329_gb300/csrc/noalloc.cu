@@ -129,7 +129,7 @@ int mgct_project_residual_static(const mgct_geom *g, int level, int view0, int n
     // transposed volume in full, one partial per projector block
     MGCT_TRY(launch_transpose_xy<float>(L.n, vol, volT, s));
     int nb = 0;
-    EpiResidual<float> e{out, b, part, L.nu, L.nv, nviews};
+    EpiResidual<float> e{out, b, part, L.nu, L.nv, nviews, {}};
     MGCT_TRY(launch_project<float>(g, level, view0, nviews, stride, vol, volT, e, s, &nb));
     return launch_sum_partials(part, nb, 1, sumsq, s);
 }

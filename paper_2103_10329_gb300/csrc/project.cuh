@@ -289,22 +289,42 @@ struct EpiPlus {
     }
 };
 
+// Where element (jv, ju) of view i of a weighted sinogram lies.  In float32 on
+// separable geometries it is [view][u][v], since the back-projector reads down
+// the detector columns (and the projector's lanes are the rows), with SINO_PAD
+// zero rows before every column and after the last; otherwise [view][v][u].
+struct SinoStrides {
+    int u, v;
+    size_t view, first;
+    __device__ size_t at(int i, int jv, int ju) const {
+        return first + (size_t)i * view + (size_t)jv * v + (size_t)ju * u;
+    }
+};
+inline bool columns_padded(const mgct_geom *g, size_t elem) { return g->separable && elem != 2; }
+inline SinoStrides weighted_strides(const mgct_geom *g, const LevelInfo &L, size_t elem) {
+    const int pitch = L.nv + SINO_PAD;
+    return columns_padded(g, elem) ? SinoStrides{pitch, 1, (size_t)L.nu * pitch, SINO_PAD}
+                                   : SinoStrides{1, L.nu, (size_t)L.nu * L.nv, 0};
+}
+
 // r = b - A vol and the block's sum of r^2 (float64) into part[block].
 // WEIGHTED = false: out = r.  WEIGHTED = true: out = r * dlh (the ray's path
-// length per plane), which the back-projector then need not recompute.
+// length per plane), which the back-projector then need not recompute, at
+// the strides ws.
 template <typename OT, bool WEIGHTED = false>
 struct EpiResidual {
     OT *out;
-    const float *b;  // indexed like out
+    const float *b;  // [i][v][u]
     double *part;    // NULL: no norm
     int nu, nv, nviews;
+    SinoStrides ws;
     __device__ void operator()(int i, int, int jv, int ju, bool active, float acc, float dlh) const {
         double s[1] = {0.0};
         if (active) {
             size_t idx = ((size_t)i * nv + jv) * nu + ju;
             float r = __ldg(b + idx) - acc * dlh;
             if (WEIGHTED) {
-                out[idx] = from_f32<OT>(r * dlh);
+                out[ws.at(i, jv, ju)] = from_f32<OT>(r * dlh);
                 s[0] = (double)r * (double)r;
             } else {
                 OT ro = from_f32<OT>(r);
@@ -329,10 +349,11 @@ struct EpiDualDot {
     const RT *rw;
     double *part;  // [blocks][2]
     int nu, nv, nviews;
+    SinoStrides ws;
     __device__ void operator()(int i, int, int jv, int ju, bool active, float acc, float dlh) const {
         double s[2] = {0.0, 0.0};
         if (active) {
-            float rv = to_f32(rw[((size_t)i * nv + jv) * nu + ju]);
+            float rv = to_f32(rw[ws.at(i, jv, ju)]);
             float ad = acc * dlh;
             s[0] = (double)rv * (double)acc;
             s[1] = (double)ad * (double)ad;
@@ -350,12 +371,13 @@ struct EpiDualDot {
 // OS-EMTR (Eq. 3) sinogram terms for one subset, weighted by dlh:
 //   t = exp(-A mu);  c0 = (t - exp(-b)) dlh  (I/I0 = exp(-b));  c1 = t PI dlh
 // b and PI are full [K][nv][nu] arrays indexed by the view k; c is a batch
-// two-channel sinogram [i][v][u][2].
+// two-channel sinogram at the strides ws.
 struct EpiEMTerms {
     float2 *c;
     const float *b;
     const float *pi;
     int nu, nv, nviews;
+    SinoStrides ws;
     __device__ void operator()(int i, int k, int jv, int ju, bool active, float acc, float dlh) const {
         if (!active) return;
         size_t pix = (size_t)jv * nu + ju;
@@ -364,7 +386,7 @@ struct EpiEMTerms {
         float2 o;
         o.x = (t - expf(-__ldg(b + full))) * dlh;
         o.y = t * __ldg(pi + full) * dlh;
-        c[(size_t)i * nv * nu + pix] = o;
+        c[ws.at(i, jv, ju)] = o;
     }
 };
 
@@ -487,7 +509,7 @@ __device__ __forceinline__ RaySum column_rays(const ProjArgs &a, const float4 *_
                                               ColTab<typename ZElem<VT, LAYOUT>::type> *__restrict__ tab) {
     using E = typename ZElem<VT, LAYOUT>::type;
     // {ax, rb, rb_lo, pb}, {pb_lo, ez0, ez0_lo, ezc}, {ezc_lo, e10, e10_lo, e1c}, {e1c_lo, 0, 0, 0}
-    const float4 t0 = __ldg(ct), t1 = __ldg(ct + 1), t2 = __ldg(ct + 2), t3 = __ldg(ct + 3);
+    const float4 t0 = __ldg(ct), t1 = __ldg(ct + a.nu), t2 = __ldg(ct + 2 * a.nu), t3 = __ldg(ct + 3 * a.nu);
     const DF rb{t0.y, t0.z}, pb{t0.w, t1.x}, ez0{t1.y, t1.z}, ezc{t1.w, t2.x}, e10{t2.y, t2.z}, e1c{t2.w, t3.x};
     const E *__restrict__ base = t0.x != 0.0f ? zqy : zqx;
     const int n = a.n, lane = threadIdx.x & 31;
@@ -600,7 +622,7 @@ __global__ void __launch_bounds__(PC_COLS *PC_ROWS, MGCT_PC_MINB)
     const bool active = view_ok && ju < a.nu && jv < a.nv;
     RaySum rs{0.0f, 0.0f};
     if (view_ok && ju < a.nu)  // uniform over the warp
-        rs = column_rays<VT, LAYOUT>(a, cols + ((size_t)k * a.nu + ju) * 4, jv, jv < a.nv, zqy, zqx,
+        rs = column_rays<VT, LAYOUT>(a, cols + (size_t)k * 4 * a.nu + ju, jv, jv < a.nv, zqy, zqx,
                                      tab[threadIdx.y]);
     epi(i, k, jv, ju, active, rs.acc, rs.dlh);
 }

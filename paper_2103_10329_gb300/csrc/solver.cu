@@ -33,6 +33,7 @@ int launch_column_table_df(const mgct_geom *g, int level, cudaStream_t s) {
     const int K = g->desc.n_views;
     const int total = K * L.nu;
     MGCT_KERNEL(KK_OTHER, s, k_column_table_df<<<(total + 255) / 256, 256, 0, s>>>(L.d_views, K, L.nu, L.d_cols_df));
+    MGCT_KERNEL(KK_OTHER, s, k_class_ranges<<<(K + 7) / 8, 256, 0, s>>>(L.d_cols_df, K, L.nu, L.d_ranges));
     return MGCT_OK;
 }
 
@@ -77,7 +78,7 @@ struct LWSpace {
 static LWSpace carve_lw(const mgct_geom *g, int level, Carver &c) {
     const LevelInfo &L = g->lev[level];
     LWSpace w;
-    w.r = c.take<float>(sino_elems(g, L));
+    w.r = c.take<float>(padded_sino_elems(g->desc.n_views, L.nu, L.nv));
     w.grad = c.take<float>(vox(L));
     w.d = c.take<float>(vox(L));
     w.muT = c.take<float>(vox(L));
@@ -97,7 +98,7 @@ struct EMSpace {
 static EMSpace carve_em(const mgct_geom *g, int level, Carver &c) {
     const LevelInfo &L = g->lev[level];
     EMSpace w;
-    w.c2 = c.take<float2>(sino_elems(g, L));  // worst case: one subset holding every view
+    w.c2 = c.take<float2>(padded_sino_elems(g->desc.n_views, L.nu, L.nv));  // worst case: one subset holding every view
     w.nd = c.take<float>(2 * vox(L));
     w.muT = c.take<float>(vox(L));
     w.part = c.take<double>(1024);
@@ -180,8 +181,9 @@ static int lw_direction(const mgct_geom *g, int level, const float *mu, const fl
     constexpr bool F32 = std::is_same<ST, float>::value;
     MGCT_TRY(check_cuda(cudaMemsetAsync(w.sums, 0, 8 * sizeof(double), s), "memset"));
     ST *r = reinterpret_cast<ST *>(w.r);
+    if (columns_padded(g, sizeof(ST))) MGCT_TRY(launch_zero_pads((size_t)K * L.nu, L.nv, sizeof(ST), r, s));
     int nb = 0;
-    EpiResidual<ST, true> er{r, b, w.part, L.nu, L.nv, K};
+    EpiResidual<ST, true> er{r, b, w.part, L.nu, L.nv, K, weighted_strides(g, L, sizeof(ST))};
     (void)F32;
     MGCT_TRY(project_quads<ST>(g, level, mu, w.muT, w.quads, er, s, &nb));
     (void)nv3;
@@ -206,7 +208,7 @@ static int lw_line_search(const mgct_geom *g, int level, const float *dir, float
     const int K = g->desc.n_views;
     const size_t nv3 = vox(L);
     int nb = 0;
-    EpiDualDot<ST> ed{reinterpret_cast<ST *>(w.r), w.part, L.nu, L.nv, K};
+    EpiDualDot<ST> ed{reinterpret_cast<ST *>(w.r), w.part, L.nu, L.nv, K, weighted_strides(g, L, sizeof(ST))};
     MGCT_TRY(project_quads<ST>(g, level, dir, spare, w.quads, ed, s, &nb));
     (void)nv3;
     return launch_sum_partials(w.part, nb, 2, w.sums + slot, s);
@@ -288,17 +290,17 @@ static int osemtr(const mgct_geom *g, int level, int M, float *mu, const float *
     EMSpace w = carve_em(g, level, c);
     const int K = g->desc.n_views;
     const size_t nv3 = vox(L);
+    if (columns_padded(g, sizeof(float2))) MGCT_TRY(launch_zero_pads((size_t)((K + M - 1) / M) * L.nu, L.nv, sizeof(float2), w.c2, s));
     for (int m = 0; m < M; ++m) {
         int cnt = (K - m + M - 1) / M;
         if (cnt <= 0) continue;
         MGCT_TRY(launch_transpose_xy<float>(L.n, mu, w.muT, s));
-        EpiEMTerms e{w.c2, b, pi, L.nu, L.nv, cnt};
+        EpiEMTerms e{w.c2, b, pi, L.nu, L.nv, cnt, weighted_strides(g, L, sizeof(float2))};
         MGCT_TRY(launch_project<float>(g, level, m, cnt, M, mu, w.muT, e, s));
-        // c2 holds room for every view; past this subset's views it is free
-        const size_t used = (size_t)cnt * L.nu * L.nv;
+        // c2 holds room for every view; past the largest subset's views it is free
+        const size_t all = padded_sino_elems(K, L.nu, L.nv), used = padded_sino_elems((K + M - 1) / M, L.nu, L.nv);
         MGCT_TRY(launch_backproject<2, float2, true>(g, level, m, cnt, M, w.c2, w.nd, 0, s,
-                                                     reinterpret_cast<float *>(w.c2 + used),
-                                                     2 * (sino_elems(g, L) - used)));
+                                                     reinterpret_cast<float *>(w.c2 + used), 2 * (all - used)));
         MGCT_TRY(launch_em_update(nv3, mu, w.nd, w.part, s));
     }
     return MGCT_OK;
@@ -326,7 +328,7 @@ static int multigrid_level(const mgct_geom *g, int level, float *mu, const MGSpa
             Carver cw(m.lw_base);
             LWSpace w = carve_lw(g, 0, cw);
             int nb = 0;
-            EpiResidual<float, false> er{w.r, b, nullptr, F.nu, F.nv, K};
+            EpiResidual<float, false> er{w.r, b, nullptr, F.nu, F.nv, K, {}};
             MGCT_TRY(project_quads<float>(g, level, mu, w.muT, w.quads, er, s, &nb));
             MGCT_TRY(launch_restrict_sino(K, F.nv, F.nu, w.r, m.bf[level + 1], s));
             trace_tag(level + 1);
@@ -406,7 +408,7 @@ int mgct_project(const mgct_geom *g, int level, int view0, int nviews, int strid
         const VT *v = static_cast<const VT *>(vol);
         VT *vT = static_cast<VT *>(g->d_scratch_vol);
         if (b) {
-            EpiResidual<OT> e{static_cast<OT *>(out), b, part, L.nu, L.nv, nviews};
+            EpiResidual<OT> e{static_cast<OT *>(out), b, part, L.nu, L.nv, nviews, {}};
             return project_volume<VT, VT>(g, level, view0, nviews, stride, v, vT, g->d_scratch_quads, e, s, &nb);
         }
         EpiStore<OT> e{static_cast<OT *>(out), L.nu, L.nv};

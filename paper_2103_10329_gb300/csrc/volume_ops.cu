@@ -738,6 +738,26 @@ __global__ void k_copy(size_t count, const float4 *__restrict__ in, float4 *__re
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < count; t += (size_t)gridDim.x * blockDim.x) out[t] = in[t];
 }
 
+// Zero rows of a weighted sinogram, one thread per column (the first also
+// those before it).
+template <typename T>
+__global__ void k_zero_pads(size_t columns, int nv, T *__restrict__ sino) {
+    for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c <= columns; c += (size_t)gridDim.x * blockDim.x) {
+        T *p = sino + (c == 0 ? 0 : c * (nv + SINO_PAD));
+        for (int j = 0; j < SINO_PAD; ++j) p[j] = T();
+    }
+}
+
+int launch_zero_pads(size_t columns, int nv, int elem, void *sino, cudaStream_t s) {
+    const int nb = grid_for(columns + 1);
+    if (elem == 4) {
+        MGCT_KERNEL(KK_UPDATE, s, k_zero_pads<uint32_t><<<nb, 256, 0, s>>>(columns, nv, static_cast<uint32_t *>(sino)));
+    } else {
+        MGCT_KERNEL(KK_UPDATE, s, k_zero_pads<uint64_t><<<nb, 256, 0, s>>>(columns, nv, static_cast<uint64_t *>(sino)));
+    }
+    return MGCT_OK;
+}
+
 int launch_copy(size_t count, const float *in, float *out, cudaStream_t s) {
     if (count % 4) return set_error(MGCT_ESHAPE, "copy size must be a multiple of 4");
     MGCT_KERNEL(KK_UPDATE, s, k_copy<<<grid_for(count / 4), 256, 0, s>>>(count / 4, reinterpret_cast<const float4 *>(in), reinterpret_cast<float4 *>(out)));
