@@ -301,6 +301,6 @@ int launch_build_zpairs(int n, const SRC *src, void *dst, cudaStream_t s);
 template <typename T>
 int launch_transpose_xy(int n, const T *in, T *out, cudaStream_t s);
 
-int launch_sum_partials(const double *part, int count, int nvals, double *out, cudaStream_t s);
+int launch_sum_partials(double *part, int count, int nvals, double *out, cudaStream_t s);
 
 }  // namespace mgct

@@ -570,8 +570,49 @@ __global__ void __launch_bounds__(1024) k_sum_partials(const double *__restrict_
     }
 }
 
-int launch_sum_partials(const double *part, int count, int nvals, double *out, cudaStream_t s) {
-    MGCT_KERNEL(KK_REDUCE, s, k_sum_partials<<<1, 1024, 0, s>>>(part, count, nvals, out));
+// First stage for long lists: block j sums entries [j SP_CHUNK, (j + 1)
+// SP_CHUNK) of each value in the same order and leaves the sums in the
+// chunk's first entry (it alone reads the chunk).
+constexpr int SP_CHUNK = 8192;
+__global__ void __launch_bounds__(256) k_sum_chunks(double *part, int count, int nvals) {
+    __shared__ double red[8];
+    const int c0 = blockIdx.x * SP_CHUNK, c1 = min(count, c0 + SP_CHUNK);
+    double total[2] = {0.0, 0.0};
+    for (int c = 0; c < nvals; ++c) {
+        double s = 0.0;
+        for (int i = c0 + threadIdx.x; i < c1; i += 256) s += part[(size_t)i * nvals + c];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = s;
+        __syncthreads();
+        if (threadIdx.x == 0)
+            for (int w = 0; w < 8; ++w) total[c] += red[w];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0)
+        for (int c = 0; c < nvals; ++c) part[(size_t)c0 * nvals + c] = total[c];
+}
+// Second stage: one warp per value over the chunks' sums.
+__global__ void k_sum_chunk_heads(const double *__restrict__ part, int chunks, int nvals, double *__restrict__ out) {
+    const int c = threadIdx.x / 32, lane = threadIdx.x % 32;
+    double s = 0.0;
+    for (int j = lane; j < chunks; j += 32) s += part[(size_t)j * SP_CHUNK * nvals + c];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) out[c] = s;
+}
+
+// Sums of `count` entries of nvals (1 or 2) interleaved values; `part` is
+// consumed.  One block for short lists; one block over 1.6e6 entries (512^3 /
+// 1440 views) took 0.97 ms a list, the two stages 0.02.
+int launch_sum_partials(double *part, int count, int nvals, double *out, cudaStream_t s) {
+    if (count <= SP_CHUNK) {
+        MGCT_KERNEL(KK_REDUCE, s, k_sum_partials<<<1, 1024, 0, s>>>(part, count, nvals, out));
+        return MGCT_OK;
+    }
+    const int chunks = (count + SP_CHUNK - 1) / SP_CHUNK;
+    MGCT_KERNEL(KK_REDUCE, s, k_sum_chunks<<<chunks, 256, 0, s>>>(part, count, nvals));
+    MGCT_KERNEL(KK_REDUCE, s, k_sum_chunk_heads<<<1, 32 * nvals, 0, s>>>(part, chunks, nvals, out));
     return MGCT_OK;
 }
 
@@ -656,19 +697,25 @@ __global__ void k_max_partials(size_t count, const float *__restrict__ x, double
     if (threadIdx.x == 0) part[blockIdx.x] = (double)red[0];
 }
 
-__global__ void k_em_update(size_t count, float *__restrict__ mu, const float *__restrict__ nd,
-                            const double *__restrict__ part, int nparts) {
-    __shared__ float thr;
-    if (threadIdx.x == 0) {
-        double m = 0.0;
-        for (int i = 0; i < nparts; ++i) m = fmax(m, part[i]);
-        thr = (float)(1e-12 * m);
-    }
+// Every block takes the maximum of the (at most 4 x 256) partials itself, by
+// all its threads: a serial loop over them in one thread held each block for
+// 0.5 ms, 4.4 of the 9.9 ms of a pass at 128^3 / 360 views (now 0.12).
+__global__ void __launch_bounds__(256) k_em_update(size_t count, float *__restrict__ mu, const float *__restrict__ nd,
+                                                   const double *__restrict__ part, int nparts) {
+    __shared__ double red[8];
+    double m = 0.0;
+    for (int i = threadIdx.x; i < nparts; i += 256) m = fmax(m, part[i]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = m;
     __syncthreads();
-    const float th = thr;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) m = fmax(m, red[w]);
+    const float th = (float)(1e-12 * m);
+    if (!(th > 0.0f)) return;
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < count; t += (size_t)gridDim.x * blockDim.x) {
         float den = nd[count + t];
-        if (den > th && th > 0.0f) mu[t] += nd[t] / den;
+        if (den > th) mu[t] += nd[t] / den;
     }
 }
 
