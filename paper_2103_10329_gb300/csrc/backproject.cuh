@@ -678,6 +678,350 @@ __global__ void __launch_bounds__(32 * BT_WARPS, PlaneTile<NCH, NP>::MIN_BLOCKS)
     }
 }
 
+// Tilted detectors (turned about their normal by up to TILT_MAX), weighted
+// sinogram stored [view][u][v].  As in the plane kernel a warp owns W voxel
+// columns of one voxel-centre plane over 32 heights, its lanes the heights, and
+// takes the detector columns 32 at a time, a lane per column for their set-up.
+// With tilt a column's rays cross the plane at positions b that drift with the
+// row, so each lane finds its own voxel columns and adds to them in shared
+// memory (no other lane has its height).
+//
+// At fixed plane and column both coordinates of the crossing are quotients of
+// affine functions of the row with the same denominator w_a.  With r rows from
+// the anchor row (nearest the tile's middle height), k = Ev_a / w_a and
+// s = r / (1 + k r) = r + d,
+//   z = z_A + s sz,   b = b_A + s sb,
+// where z_A, b_A and the slope sz come from the view table in double-float
+// and d = -k r^2 / (1 + k r) is a small correction: the height above a lane's
+// z keeps its digits (r sz - z in one rounding), a weight is accurate to a few
+// 1e-7.  A lane's first row is the ceiling of the inverse, r = s / (1 - k s),
+// at height z - 1.
+//
+// A height's tent holds at most 4 rows where sz > 1/2, and these fall into at
+// most 3 neighbouring voxel columns where 3 sb < 1: a lane adds 3 sums per
+// column.  5 rows with a test of each ray's major axis serve sz > 0.4 and
+// columns that hold rays of both classes; other steps and strong drifts go
+// row by row, each ray set up in double-float as the projector sets it up.
+//
+// The per-voxel gather (k_backproject), which does that for every candidate
+// pixel of a voxel, took 128 ms at 128^3 / 192^2 / 360 views (about 6000
+// instructions a voxel, view and warp); this kernel 5.7 ms, bound by issue.
+template <int NCH>
+struct TiltTile {
+    static constexpr int W = NCH == 2 ? 8 : 16, ZT = 32, ZP = ZT + 1;
+    static constexpr int ROWS = W + 4;  // voxel columns b0 - 2 .. b0 + W + 1 (the outer ones are dropped)
+};
+
+struct __align__(16) TiltEntry {
+    float sz, szlo;   // height step per row at the anchor
+    float d1, rz;     // 1 + height of the anchor row above the tile's middle; 1 / sz
+    float k, sb;      // Ev_a / w_a; step along b per row at the anchor
+    float bA;         // anchor row's b from the tile's edge
+    int jv;           // anchor row
+    long long base;   // element of the column's row 0
+    int i, ju;        // view of the batch and column
+};
+
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float2 tl_row(const float *p, float w) { return make_float2(ld_if(p, w), 0.0f); }
+__device__ __forceinline__ float2 tl_row(const float2 *p, float w) { return bt_row(p, p, 0, both(w)); }
+
+// Which classes the rays of a detector column may have (bit 0: x-major, bit 1:
+// y-major): y-major where (w_y - w_x) (w_y + w_x) > 0, both factors affine in
+// the row; both classes where a factor changes sign over the detector or
+// comes within rounding of 0, otherwise the projector's own choice.
+__device__ __forceinline__ int column_classes(const ViewGeom &G, float up, float cv) {
+    const RayDir d0 = ray_dir(G, up, -cv), d1 = ray_dir(G, up, cv);
+    const float eps = 1e-5f * (fabsf(d0.wx) + fabsf(d0.wy) + fabsf(d1.wx) + fabsf(d1.wy));
+    const float a0 = d0.wy - d0.wx, a1 = d1.wy - d1.wx, b0 = d0.wy + d0.wx, b1 = d1.wy + d1.wx;
+    const bool same = (fminf(a0, a1) > eps || fmaxf(a0, a1) < -eps) && (fminf(b0, b1) > eps || fmaxf(b0, b1) < -eps);
+    return same ? 1 << d0.ax : 3;
+}
+
+// A ray's crossing of the plane at c_a of its axis ax, centred, and 1 / w_a, in
+// double-float from the projector's own quantities.
+__device__ __forceinline__ void ray_crossing(const ViewGeom &G, int ax, float up, float vp, float ca, DF &xb, DF &xz,
+                                             DF &rwa) {
+    const int ib = 1 - ax;
+    const DF wa = df_affine(G.Wc[ax], G.Wc_lo[ax], G.Eu[ax], G.Eu_lo[ax], G.Ev[ax], G.Ev_lo[ax], up, vp);
+    const DF wb = df_affine(G.Wc[ib], G.Wc_lo[ib], G.Eu[ib], G.Eu_lo[ib], G.Ev[ib], G.Ev_lo[ib], up, vp);
+    const DF wz = df_affine(G.Wc[2], G.Wc_lo[2], G.Eu[2], G.Eu_lo[2], G.Ev[2], G.Ev_lo[2], up, vp);
+    const float *N = ax ? G.NY : G.NX, *Nl = ax ? G.NY_lo : G.NX_lo;
+    const DF nb = df_affine(N[0], Nl[0], N[1], Nl[1], N[2], Nl[2], up, vp);
+    const DF nz = df_affine(N[3], Nl[3], N[4], Nl[4], N[5], Nl[5], up, vp);
+    rwa = df_div(DF{1.0f, 0.0f}, wa);
+    xb = df_mul(df_add(nb, df_mul_f(wb, ca)), rwa);
+    xz = df_mul(df_add(nz, df_mul_f(wz, ca)), rwa);
+}
+
+template <int NCH, typename ST>
+__global__ void __launch_bounds__(32 * BT_WARPS, 3)
+    k_backproject_tilt(BPArgs a, const int2 *__restrict__ ranges, const ST *__restrict__ sino, float *__restrict__ out,
+                       int accumulate) {
+    using T = TiltTile<NCH>;
+    constexpr int W = T::W, ZT = T::ZT, ZP = T::ZP;
+    __shared__ TiltEntry tabs[BT_WARPS][32];
+    __shared__ float acc[BT_WARPS][NCH][T::ROWS][ZP];
+    constexpr unsigned FULL = 0xffffffffu;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // parts, classes, planes and tiles as in k_backproject_plane
+    const int parts = a.splits * (a.cls < 0 ? 2 : 1);
+    const int ztiles = gridDim.z / parts;
+    const int part = blockIdx.z / ztiles;
+    const int z0 = (blockIdx.z - part * ztiles) * ZT;
+    const int cls = a.cls < 0 ? part / a.splits : a.cls;
+    const int split = part - (a.cls < 0 ? cls * a.splits : 0);
+    const int per = (a.nviews + a.splits - 1) / a.splits;
+    const int i0 = split * per, i1 = min(a.nviews, i0 + per);
+    const int p0 = blockIdx.y * BT_WARPS, pl = p0 + warp, b0 = blockIdx.x * W;
+    const float ic = 0.5f * (float)(a.n - 1);
+    const float cu = 0.5f * (float)(a.nu - 1), cv = 0.5f * (float)(a.nv - 1);
+    const float ca = (float)pl - ic, cb0 = (float)b0 - ic;
+    const float zc = (float)(z0 + ZT / 2) - ic;  // the tile's middle height, centred (exact)
+    const float zl = (float)(lane - ZT / 2);
+    const int pitch = a.nv + SINO_PAD;
+    TiltEntry *tab = tabs[warp];
+    float(*accw)[T::ROWS][ZP] = acc[warp];
+#pragma unroll
+    for (int q = 0; q < NCH; ++q)
+        for (int r = 0; r < T::ROWS; ++r) accw[q][r][lane] = 0.0f;
+
+    for (int ib = i0; ib < i1 && pl < a.n; ib += 32) {
+        // lane = view: the columns of the tile's piece of the plane, a voxel
+        // wider all round: between the projections of its corners
+        int vlo = 0, cnt = 0;
+        if (ib + lane < i1) {
+            const int k = a.view0 + (ib + lane) * a.stride;
+            const ViewGeom &G = a.views[k];
+            float lo = 1e30f, hi = -1e30f;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float b = (float)(c & 1 ? min(b0 + W, a.n) : b0 - 1);
+                const float Z = (float)(c & 2 ? min(z0 + ZT, a.n) : z0 - 1) - G.S[2];
+                const float X = (cls ? b : (float)pl) - G.S[0], Y = (cls ? (float)pl : b) - G.S[1];
+                const float q0 = fmaf(G.Q[2], Z, fmaf(G.Q[1], Y, G.Q[0] * X));
+                const float q2 = fmaf(G.Q[8], Z, fmaf(G.Q[7], Y, G.Q[6] * X));
+                const float u = q0 / q2 + cu;
+                lo = fminf(lo, u);
+                hi = fmaxf(hi, u);
+            }
+            const int2 r = __ldg(ranges + 2 * k + cls);
+            vlo = max(r.x, (int)ceilf(lo - 1e-2f));
+            cnt = max(0, min(r.y, (int)floorf(hi + 1e-2f)) - vlo + 1);
+        }
+        int pre = cnt;  // the views' columns as one list
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(FULL, pre, o);
+            if (lane >= o) pre += v;
+        }
+        const int total = __shfl_sync(FULL, pre, 31);
+        for (int first = 0; __any_sync(FULL, first < total); first += 32) {
+            const int idx = first + lane;
+            int v = 0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(FULL, pre, v + o - 1) <= idx) v += o;
+            const int ju = __shfl_sync(FULL, vlo, v & 31) + idx - __shfl_sync(FULL, pre - cnt, v & 31);
+            bool ok = idx < total;
+            int form = 2;  // 0: 4 rows of one class, 1: 5 rows and a class test, 2: row by row
+            TiltEntry t;
+            if (ok) {
+                t.i = ib + v;
+                t.ju = ju;
+                t.base = (long long)SINO_PAD + ((long long)t.i * a.nu + ju) * pitch;
+                const ViewGeom &G = a.views[a.view0 + t.i * a.stride];
+                const float up = (float)ju - cu;
+                const float *N = cls ? G.NY : G.NX, *Nl = cls ? G.NY_lo : G.NX_lo;
+                const int classes = column_classes(G, up, cv);
+                ok = (classes >> cls) & 1;
+                // height (e0 + v' e1) / (w0 + v' w1): the anchor row, any row near it will do
+                const float w0 = fmaf(up, G.Eu[cls], G.Wc[cls]), w1 = G.Ev[cls];
+                const float e0 = fmaf(up, N[4], N[3]) + ca * fmaf(up, G.Eu[2], G.Wc[2]), e1 = fmaf(ca, G.Ev[2], N[5]);
+                const float jf = rintf((zc * w0 - e0) / (e1 - zc * w1) + cv);
+                DF xb, xz, rwa2;
+                ray_crossing(G, cls, up, jf - cv, ca, xb, xz, rwa2);
+                const DF va{G.Ev[cls], G.Ev_lo[cls]};
+                const DF dz = df_add(df_add(DF{N[5], Nl[5]}, df_mul_f(DF{G.Ev[2], G.Ev_lo[2]}, ca)),
+                                     df_mul(DF{-xz.hi, -xz.lo}, va));
+                const DF sz = df_mul(dz, rwa2);
+                const float rwa = rwa2.hi;
+                const DF da = df_add(xz, DF{-zc, 0.0f}), ba = df_add(xb, DF{-cb0, 0.0f});
+                t.sz = sz.hi;
+                t.szlo = sz.lo;
+                t.rz = 1.0f / sz.hi;
+                t.d1 = __fadd_rn(da.hi, 1.0f) + da.lo;
+                t.k = va.hi * rwa;
+                t.sb = (fmaf(ca, G.Ev[1 - cls], N[2]) - xb.hi * va.hi) * rwa;
+                t.bA = ba.hi + ba.lo;
+                t.jv = (int)jf;
+                // over the tile's rows the steps differ from the anchor's by at
+                // most (1 + kr)^2
+                const float kr = fabsf(t.k) * (fabsf(t.d1) + (float)ZT) * t.rz;
+                const float smin = t.sz / ((1.0f + kr) * (1.0f + kr)), bmax = fabsf(t.sb) / ((1.0f - kr) * (1.0f - kr));
+                if (fabsf(jf) < 1.0e6f && kr < 0.25f) {
+                    if (smin > 0.501f && bmax < 0.3f && classes != 3) form = 0;
+                    else if (smin > 0.401f && bmax < 0.22f) form = 1;
+                }
+                if (ok && form < 2) {
+                    // columns whose rows at the tile's heights all lie off the detector
+                    const float sa = ((float)(-ZT / 2) - t.d1) * t.rz, sb = ((float)(ZT / 2) + 1.0f - t.d1) * t.rz;
+                    const float ra = sa / (1.0f - t.k * sa) + jf, rb = sb / (1.0f - t.k * sb) + jf;
+                    ok = ra < (float)a.nv + 1.0f && rb > -2.0f;
+                }
+            }
+            // the table, ordered by form
+            const unsigned below = (1u << lane) - 1u;
+            int end[3], run = 0;
+#pragma unroll
+            for (int f = 0; f < 3; ++f) {
+                const unsigned m = __ballot_sync(FULL, ok && form == f);
+                if (ok && form == f) tab[run + __popc(m & below)] = t;
+                run += __popc(m);
+                end[f] = run;
+            }
+            __syncwarp();
+            auto rows = [&](const TiltEntry &c, auto ntag) {
+                constexpr int R = decltype(ntag)::value;
+                const float s1 = (zl - c.d1) * c.rz, ks = c.k * s1;
+                const float r0 = __fadd_ru(fmaf(ks * s1, rcp_approx(1.0f - ks), s1), BT_MAGIC) - BT_MAGIC;
+                const int row = (int)r0 + c.jv;
+                const ST *p = sino + c.base + row;
+                float w[R], b[R];
+                float2 y[R];
+                // R = 5: the projector's axis choice, ray by ray (ray_dir's own operations)
+                float cx = 0.0f, cy = 0.0f, vx = 0.0f, vy = 0.0f;
+                if (R == 5) {
+                    const ViewGeom &G = a.views[a.view0 + c.i * a.stride];
+                    const float up = (float)c.ju - cu;
+                    cx = __fmaf_rn(up, G.Eu[0], G.Wc[0]);
+                    cy = __fmaf_rn(up, G.Eu[1], G.Wc[1]);
+                    vx = G.Ev[0];
+                    vy = G.Ev[1];
+                }
+#pragma unroll
+                for (int s = 0; s < R; ++s) {
+                    const float r = r0 + (float)s, kr = c.k * r;
+                    const float d = -(kr * r) * rcp_approx(1.0f + kr);
+                    const float g = fmaf(r, c.sz, -zl) + fmaf(d, c.sz, fmaf(r, c.szlo, c.d1));
+                    b[s] = fmaf(d, c.sb, fmaf(r, c.sb, c.bA));
+                    bool in = (unsigned)(row + s) < (unsigned)a.nv;
+                    if (R == 5) {
+                        const float vp = (float)(row + s) - cv;
+                        in = in && (fabsf(__fmaf_rn(vp, vy, cy)) > fabsf(__fmaf_rn(vp, vx, cx))) == (cls != 0);
+                    }
+                    w[s] = in ? 1.0f - fabsf(g - 1.0f) : -1.0f;
+                    y[s] = tl_row(p + s, w[s]);
+                }
+                const float bl = floorf(fminf(b[0], b[R - 1]));
+                float2 p0 = both(0.0f), p1 = both(0.0f), p2 = both(0.0f);  // voxel columns bl, bl + 1, bl + 2
+#pragma unroll
+                for (int s = 0; s < R; ++s) {
+                    const float q = b[s] - bl - 1.0f, qm = 1.0f - fabsf(q);  // q in [-1, 1)
+                    const float2 wy = make_float2(w[s] * y[s].x, NCH == 2 ? w[s] * y[s].y : 0.0f);
+                    p1 = fma_f2(both(qm), wy, p1);
+                    if (q < 0.0f) p0 = fma_f2(both(-q), wy, p0);
+                    if (q > 0.0f) p2 = fma_f2(both(q), wy, p2);
+                }
+                const int j = (int)bl;
+                if ((unsigned)(j + 2) < (unsigned)(W + 2)) {
+                    float *d = &accw[0][j + 2][lane];
+                    d[0] += p0.x;
+                    d[ZP] += p1.x;
+                    d[2 * ZP] += p2.x;
+                    if (NCH == 2) {
+                        d = &accw[NCH - 1][j + 2][lane];
+                        d[0] += p0.y;
+                        d[ZP] += p1.y;
+                        d[2 * ZP] += p2.y;
+                    }
+                }
+            };
+            for (int e = 0; e < end[0]; ++e) rows(tab[e], std::integral_constant<int, 4>());
+            for (int e = end[0]; e < end[1]; ++e) rows(tab[e], std::integral_constant<int, 5>());
+            for (int e = end[1]; e < end[2]; ++e) {
+                const TiltEntry &c = tab[e];
+                const ViewGeom &G = a.views[a.view0 + c.i * a.stride];
+                const float up = (float)c.ju - cu, cz = (float)(z0 + lane) - ic;
+                const float *N = cls ? G.NY : G.NX;
+                const float w0 = fmaf(up, G.Eu[cls], G.Wc[cls]), w1 = G.Ev[cls];
+                const float e0 = fmaf(up, N[4], N[3]) + ca * fmaf(up, G.Eu[2], G.Wc[2]), e1 = fmaf(ca, G.Ev[2], N[5]);
+                // rows at heights z - 1 and z + 1, with a row to spare
+                const float va = ((cz - 1.0f) * w0 - e0) / (e1 - (cz - 1.0f) * w1) + cv;
+                const float vb = ((cz + 1.0f) * w0 - e0) / (e1 - (cz + 1.0f) * w1) + cv;
+                const int rlo = (int)fmaxf(0.0f, floorf(fminf(va, vb)) - 1.0f);
+                const int rhi = (int)fminf((float)(a.nv - 1), ceilf(fmaxf(va, vb)) + 1.0f);
+                for (int row = rlo; row <= rhi; ++row) {
+                    const float vp = (float)row - cv;
+                    if (ray_dir(G, up, vp).ax != cls) continue;
+                    DF xb, xz, rwa;
+                    ray_crossing(G, cls, up, vp, ca, xb, xz, rwa);
+                    const float hz = 1.0f - fabsf(__fadd_rn(__fsub_rn(xz.hi, cz), xz.lo));
+                    if (!(hz > 0.0f)) continue;
+                    int j;
+                    float tb;
+                    split_coord(df_add(xb, DF{-cb0, 0.0f}), j, tb);
+                    if ((unsigned)(j + 2) >= (unsigned)(W + 2)) continue;
+                    const float2 y = tl_row(sino + c.base + row, 1.0f);
+                    const float wl = hz * (1.0f - tb), wh = hz * tb;
+                    float *d = &accw[0][j + 2][lane];
+                    d[0] = fmaf(wl, y.x, d[0]);
+                    if (wh > 0.0f) d[ZP] = fmaf(wh, y.x, d[ZP]);
+                    if (NCH == 2) {
+                        d = &accw[NCH - 1][j + 2][lane];
+                        d[0] = fmaf(wl, y.y, d[0]);
+                        if (wh > 0.0f) d[ZP] = fmaf(wh, y.y, d[ZP]);
+                    }
+                }
+            }
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    const size_t nvox = (size_t)a.n * a.n * a.n;
+    float *o = out + (size_t)part * NCH * nvox;
+    for (int t = tid; t < BT_WARPS * W * ZT; t += 32 * BT_WARPS) {
+        const int c = t % (BT_WARPS * W), zz = t / (BT_WARPS * W), z = z0 + zz;
+        const int w = cls ? c / W : c % BT_WARPS, j = cls ? c % W : c / BT_WARPS;
+        const int x = cls ? b0 + j : p0 + w, y = cls ? p0 + w : b0 + j;
+        if (x < a.n && y < a.n && z < a.n) {
+            const size_t idx = ((size_t)z * a.n + y) * a.n + x;
+#pragma unroll
+            for (int q = 0; q < NCH; ++q) {
+                float v = acc[w][q][j + 2][zz];
+                if (accumulate) v += o[idx + q * nvox];
+                o[idx + q * nvox] = v;
+            }
+        }
+    }
+}
+
+// k_class_ranges on tilted geometries: columns that may hold rays of a class.
+__global__ void k_class_ranges_tilt(const ViewGeom *__restrict__ views, int K, int nu, int nv, int2 *__restrict__ ranges) {
+    const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (k >= K) return;
+    int lo[2] = {nu, nu}, hi[2] = {-1, -1};
+    for (int u = lane; u < nu; u += 32) {
+        const int m = column_classes(views[k], (float)u - 0.5f * (float)(nu - 1), 0.5f * (float)(nv - 1));
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+            if ((m >> c) & 1) {
+                lo[c] = min(lo[c], u);
+                hi[c] = max(hi[c], u);
+            }
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        lo[c] = __reduce_min_sync(0xffffffffu, lo[c]);
+        hi[c] = __reduce_max_sync(0xffffffffu, hi[c]);
+        if (lane == 0) ranges[2 * k + c] = make_int2(lo[c], hi[c]);
+    }
+}
+
 // Double-float column table (see LevelInfo::d_cols_df), one thread per (view,
 // column): the axis choice is the projector's own ray_dir() at v' = 0; the
 // quotients by w_a are taken in double-float from the view table's
@@ -779,21 +1123,16 @@ inline int plane_splits(int resident, int blocks, int nviews, int most) {
     return best;
 }
 
-template <int NCH, int NP, typename ST>
-int launch_backproject_plane(const LevelInfo &L, BPArgs a, const ST *sino, float *out, int accumulate, cudaStream_t s,
-                             float *split_buf, size_t cap) {
-    using T = PlaneTile<NCH, NP>;
-    auto *kernel = k_backproject_plane<NCH, NP, ST>;
-    constexpr size_t smem = T::smem;
-    static_assert(smem <= 48 * 1024, "within the default shared-memory limit");
-    dim3 grid((L.n + T::W - 1) / T::W, (L.n + BT_WARPS - 1) / BT_WARPS, (L.n + T::ZT - 1) / T::ZT);
+// Launches a tile kernel (k_backproject_plane, k_backproject_tilt): both ray
+// classes and the view ranges in one launch, each into its own partial volume
+// of split_buf (cap floats), or one class after the other without one.
+template <int NCH, typename F, typename KF>
+int launch_tiles(const LevelInfo &L, BPArgs a, dim3 grid, KF kernel, size_t smem, float *out, int accumulate,
+                 cudaStream_t s, float *split_buf, size_t cap, F run) {
     const size_t vol_floats = (size_t)NCH * L.n * L.n * L.n;
     const int room = split_buf ? (int)(cap / vol_floats < 64 ? cap / vol_floats : 64) : 0;
     if (room < 2) {
-        // no room for partial volumes: the two ray classes one after the other
-        for (a.cls = 1; a.cls >= 0; --a.cls)
-            MGCT_KERNEL(KK_BACKPROJECT, s,
-                        kernel<<<grid, 32 * BT_WARPS, smem, s>>>(a, L.d_cols_df, L.d_ranges, sino, out, accumulate || a.cls == 0));
+        for (a.cls = 1; a.cls >= 0; --a.cls) MGCT_KERNEL(KK_BACKPROJECT, s, run(a, grid, out, accumulate || a.cls == 0));
         return MGCT_OK;
     }
     int dev = 0, sms = 0, occ = 0;
@@ -803,10 +1142,35 @@ int launch_backproject_plane(const LevelInfo &L, BPArgs a, const ST *sino, float
     a.splits = plane_splits(sms * (occ > 0 ? occ : 1), 2 * (int)(grid.x * grid.y * grid.z), a.nviews, room / 2);
     const int parts = 2 * a.splits;
     grid.z *= parts;
-    MGCT_KERNEL(KK_BACKPROJECT, s, kernel<<<grid, 32 * BT_WARPS, smem, s>>>(a, L.d_cols_df, L.d_ranges, sino, split_buf, 0));
+    MGCT_KERNEL(KK_BACKPROJECT, s, run(a, grid, split_buf, 0));
     const int sb = (int)((vol_floats + 255) / 256 < 4096 ? (vol_floats + 255) / 256 : 4096);
     MGCT_KERNEL(KK_BACKPROJECT, s, k_sum_parts<<<sb, 256, 0, s>>>(vol_floats, parts, split_buf, out, accumulate));
     return MGCT_OK;
+}
+
+template <int NCH, int NP, typename ST>
+int launch_backproject_plane(const LevelInfo &L, const BPArgs &a, const ST *sino, float *out, int accumulate,
+                             cudaStream_t s, float *split_buf, size_t cap) {
+    using T = PlaneTile<NCH, NP>;
+    constexpr size_t smem = T::smem;
+    static_assert(smem <= 48 * 1024, "within the default shared-memory limit");
+    const dim3 grid((L.n + T::W - 1) / T::W, (L.n + BT_WARPS - 1) / BT_WARPS, (L.n + T::ZT - 1) / T::ZT);
+    return launch_tiles<NCH>(L, a, grid, k_backproject_plane<NCH, NP, ST>, smem, out, accumulate, s, split_buf, cap,
+                             [&](const BPArgs &b, dim3 g, float *dst, int acc) {
+                                 k_backproject_plane<NCH, NP, ST>
+                                     <<<g, 32 * BT_WARPS, smem, s>>>(b, L.d_cols_df, L.d_ranges, sino, dst, acc);
+                             });
+}
+
+template <int NCH, typename ST>
+int launch_backproject_tilt(const LevelInfo &L, const BPArgs &a, const ST *sino, float *out, int accumulate,
+                            cudaStream_t s, float *split_buf, size_t cap) {
+    using T = TiltTile<NCH>;
+    const dim3 grid((L.n + T::W - 1) / T::W, (L.n + BT_WARPS - 1) / BT_WARPS, (L.n + T::ZT - 1) / T::ZT);
+    return launch_tiles<NCH>(L, a, grid, k_backproject_tilt<NCH, ST>, 0, out, accumulate, s, split_buf, cap,
+                             [&](const BPArgs &b, dim3 g, float *dst, int acc) {
+                                 k_backproject_tilt<NCH, ST><<<g, 32 * BT_WARPS, 0, s>>>(b, L.d_ranges, sino, dst, acc);
+                             });
 }
 
 // A^T of a weighted sinogram stored [view][u][v] on a separable geometry.
@@ -846,9 +1210,11 @@ int launch_backproject(const mgct_geom *g, int level, int view0, int nviews, int
                        float *out, int accumulate, cudaStream_t s, float *split_buf = nullptr, size_t cap = 0) {
     const LevelInfo &L = g->lev[level];
     const BPArgs a = bp_args(L, view0, nviews, stride);
-    if (g->separable && WEIGHTED) {
-        if constexpr (sizeof(ST) == 2) return launch_backproject16<ST>(L, a, sino, out, accumulate, s, split_buf, cap);
-        else return launch_backproject_cols<NCH, ST>(L, a, sino, out, accumulate, s, split_buf, cap);
+    if constexpr (WEIGHTED && sizeof(ST) == 2) {
+        if (g->separable) return launch_backproject16<ST>(L, a, sino, out, accumulate, s, split_buf, cap);
+    } else if constexpr (WEIGHTED) {
+        if (g->separable) return launch_backproject_cols<NCH, ST>(L, a, sino, out, accumulate, s, split_buf, cap);
+        if (columns_padded(g, sizeof(ST))) return launch_backproject_tilt<NCH, ST>(L, a, sino, out, accumulate, s, split_buf, cap);
     }
     if constexpr (!WEIGHTED) {
         if (g->separable) {
@@ -901,10 +1267,43 @@ __global__ void __launch_bounds__(256)
             w[SINO_PAD + ((size_t)i * a.nu + u0 + r) * pitch + jv] = tile[threadIdx.x][r];
 }
 
-// Runs the public A^T through k_weight_rays and the plane kernel, in chunks of
-// views that fit the quad scratch, and sets *ran; leaves *ran = 0 (nothing
-// launched) where it does not apply: tilted detectors, no views, or a
-// scratch smaller than one view.
+// The same on tilted geometries, each ray's slopes in double-float from the
+// view table.
+template <typename ST>
+__global__ void __launch_bounds__(256)
+    k_weight_rays_tilt(BPArgs a, const ST *__restrict__ sino, float *__restrict__ w) {
+    __shared__ float tile[32][33];
+    const int u0 = blockIdx.x * 32, v0 = blockIdx.y * 32, i = blockIdx.z;
+    const ViewGeom &G = a.views[a.view0 + i * a.stride];
+    const size_t base = (size_t)i * a.nv * a.nu;
+    const int pitch = a.nv + SINO_PAD;
+    const int ju = u0 + threadIdx.x;
+    if (blockIdx.x + blockIdx.y + blockIdx.z == 0 && threadIdx.y == 0 && threadIdx.x < SINO_PAD) w[threadIdx.x] = 0.0f;
+    for (int r = threadIdx.y; r < 32; r += 8) {
+        float v = 0.0f;  // the zero rows
+        if (ju < a.nu && v0 + r < a.nv) {
+            const float up = (float)ju - 0.5f * (float)(a.nu - 1), vp = (float)(v0 + r) - 0.5f * (float)(a.nv - 1);
+            const int ia = ray_dir(G, up, vp).ax, ib = 1 - ia;
+            const DF wa = df_affine(G.Wc[ia], G.Wc_lo[ia], G.Eu[ia], G.Eu_lo[ia], G.Ev[ia], G.Ev_lo[ia], up, vp);
+            const DF wb = df_affine(G.Wc[ib], G.Wc_lo[ib], G.Eu[ib], G.Eu_lo[ib], G.Ev[ib], G.Ev_lo[ib], up, vp);
+            const DF wz = df_affine(G.Wc[2], G.Wc_lo[2], G.Eu[2], G.Eu_lo[2], G.Ev[2], G.Ev_lo[2], up, vp);
+            const float rb = df_div(wb, wa).hi, rz = df_div(wz, wa).hi;
+            v = sqrtf(fmaf(rz, rz, fmaf(rb, rb, 1.0f))) * a.h * to_f32(__ldg(sino + base + (size_t)(v0 + r) * a.nu + ju));
+        }
+        tile[r][threadIdx.x] = v;
+    }
+    __syncthreads();
+    const int jv = v0 + threadIdx.x;
+    if (jv < pitch)
+        for (int r = threadIdx.y; r < 32 && u0 + r < a.nu; r += 8)
+            w[SINO_PAD + ((size_t)i * a.nu + u0 + r) * pitch + jv] = tile[threadIdx.x][r];
+}
+
+// Runs the public A^T through k_weight_rays and the plane kernel (tilted
+// detectors: their own), in chunks of views that fit the quad scratch, and
+// sets *ran; leaves *ran = 0 (nothing launched) where it does not apply:
+// detectors tilted by more than TILT_MAX, no views, or a scratch smaller than
+// one view.
 template <typename ST>
 int launch_backproject_public(const mgct_geom *g, int level, int view0, int nviews, int stride, const ST *sino,
                               float *out, int accumulate, cudaStream_t s, int *ran) {
@@ -913,7 +1312,7 @@ int launch_backproject_public(const mgct_geom *g, int level, int view0, int nvie
     const size_t view_elems = (size_t)L.nu * L.nv;
     const size_t cap = 2 * quad_elems(g->lev[0].n) * 4;  // floats in the quad scratch
     const size_t padded = (size_t)L.nu * (L.nv + SINO_PAD);  // a view of weighted rays
-    if (!g->separable || !L.d_cols_df || nviews < 1 || cap < padded + SINO_PAD || L.nv > 65535) return MGCT_OK;
+    if (!columns_padded(g, sizeof(float)) || !L.d_ranges || nviews < 1 || cap < padded + SINO_PAD || L.nv > 65535) return MGCT_OK;
     size_t chunk = (cap - SINO_PAD) / padded;
     if (chunk > (size_t)nviews) chunk = nviews;
     if (chunk > 65535) chunk = 65535;
@@ -922,12 +1321,19 @@ int launch_backproject_public(const mgct_geom *g, int level, int view0, int nvie
         const int cn = nviews - c0 < (int)chunk ? nviews - c0 : (int)chunk;
         const BPArgs a = bp_args(L, view0 + c0 * stride, cn, stride);
         const dim3 wgrid((L.nu + 31) / 32, (L.nv + SINO_PAD + 31) / 32, cn);
-        MGCT_KERNEL(KK_BACKPROJECT, s,
-                    k_weight_rays<ST><<<wgrid, dim3(32, 8), 0, s>>>(a, L.d_cols_df, sino + (size_t)c0 * view_elems, w));
         // what the weighted rays leave of the scratch holds partial volumes
         const size_t used = ((size_t)cn * padded + SINO_PAD + 63) & ~(size_t)63;
-        MGCT_TRY((launch_backproject_cols<1, float>(L, a, w, out, (accumulate || c0) ? 1 : 0, s, w + used,
-                                                    cap > used ? cap - used : 0)));
+        float *free_buf = w + used;
+        const size_t free_cap = cap > used ? cap - used : 0;
+        const ST *sc = sino + (size_t)c0 * view_elems;
+        const int acc = accumulate || c0 ? 1 : 0;
+        if (g->separable) {
+            MGCT_KERNEL(KK_BACKPROJECT, s, k_weight_rays<ST><<<wgrid, dim3(32, 8), 0, s>>>(a, L.d_cols_df, sc, w));
+            MGCT_TRY((launch_backproject_cols<1, float>(L, a, w, out, acc, s, free_buf, free_cap)));
+        } else {
+            MGCT_KERNEL(KK_BACKPROJECT, s, k_weight_rays_tilt<ST><<<wgrid, dim3(32, 8), 0, s>>>(a, sc, w));
+            MGCT_TRY((launch_backproject_tilt<1, float>(L, a, w, out, acc, s, free_buf, free_cap)));
+        }
     }
     *ran = 1;
     return MGCT_OK;

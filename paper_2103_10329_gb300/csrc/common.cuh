@@ -65,7 +65,7 @@ struct LevelInfo {
     // range of that table's z step per detector row, E1 = e10 + c_a e1c, over
     // every view, column and voxel-centre plane c_a
     float e1_lo, e1_hi;
-    int2 *d_ranges;     // device [K][2] first and last column of x-major and of y-major rays (with d_cols_df)
+    int2 *d_ranges;     // device [K][2] first and last column of x-major and of y-major rays
 };
 
 // Detector-column table of a separable geometry (no detector tilt): for view
@@ -78,6 +78,9 @@ struct LevelInfo {
 // pb}, {pb_lo, ez0, ez0_lo, ezc}, {ezc_lo, e10, e10_lo, e1c}, {e1c_lo, 0, 0,
 // 0} (centred: E0 + c_z = ez0 + c_a ezc), each an array over the columns.
 int launch_column_table_df(const mgct_geom *g, int level, cudaStream_t s);
+// d_ranges of a tilted geometry.
+int launch_class_ranges_tilt(const mgct_geom *g, int level, cudaStream_t s);
+constexpr float TILT_MAX = 0.35f;  // |Ev horizontal| / Ev_z: heights then rise with the row on every ray
 // In float32: entry {ax, rb, pb, ez0}, {ezc, e10, e1c, 0}.
 int launch_column_table(const mgct_geom *g, int level, cudaStream_t s);
 
@@ -88,6 +91,7 @@ struct mgct_geom {
     std::vector<double> theta, z, drift;
     int has_drift;
     int separable;  // 1 if no view has a tilted detector (e_u horizontal, e_v vertical)
+    int small_tilt;  // 1 if every view's detector rows lean by at most TILT_MAX from vertical
     int levels;
     mgct::LevelInfo lev[8];
     std::vector<mgct::ViewGeom> h_views[8];

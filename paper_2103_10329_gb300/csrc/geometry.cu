@@ -229,7 +229,7 @@ static void e1_range(LevelInfo &L, const std::vector<ViewGeom> &hv) {
 
 static int upload_tables(mgct_geom *g) {
     int K = g->desc.n_views;
-    g->separable = 1;
+    g->separable = g->small_tilt = 1;
     for (int l = 0; l < g->levels; ++l) {
         auto &hv = g->h_views[l];
         hv.resize(K);
@@ -241,6 +241,7 @@ static int upload_tables(mgct_geom *g) {
             if (v.Ev[0] != 0.0f || v.Ev[1] != 0.0f || v.Eu[2] != 0.0f || v.Ev_lo[0] != 0.0f ||
                 v.Ev_lo[1] != 0.0f || v.Eu_lo[2] != 0.0f || v.Q[2] != 0.0f || v.Q[8] != 0.0f)
                 g->separable = 0;
+            if (!(std::hypot((double)v.Ev[0], (double)v.Ev[1]) <= TILT_MAX * (double)v.Ev[2])) g->small_tilt = 0;
         }
         MGCT_TRY(check_cuda(cudaMemcpy(g->lev[l].d_views, hv.data(), K * sizeof(ViewGeom),
                                        cudaMemcpyHostToDevice),
@@ -248,15 +249,18 @@ static int upload_tables(mgct_geom *g) {
     }
     for (int l = 0; l < g->levels; ++l) {
         LevelInfo &L = g->lev[l];
-        if (!g->separable) continue;
+        if (!L.d_ranges)
+            MGCT_TRY(check_cuda(cudaMalloc(&L.d_ranges, (size_t)K * 2 * sizeof(int2)), "allocate column ranges"));
+        if (!g->separable) {
+            MGCT_TRY(launch_class_ranges_tilt(g, l, 0));
+            continue;
+        }
         e1_range(L, g->h_views[l]);
         if (!L.d_cols)
             MGCT_TRY(check_cuda(cudaMalloc(&L.d_cols, (size_t)K * L.nu * 2 * sizeof(float4)), "allocate column table"));
         if (!L.d_cols_df)
             MGCT_TRY(check_cuda(cudaMalloc(&L.d_cols_df, (size_t)K * L.nu * 4 * sizeof(float4)),
                                 "allocate column table"));
-        if (!L.d_ranges)
-            MGCT_TRY(check_cuda(cudaMalloc(&L.d_ranges, (size_t)K * 2 * sizeof(int2)), "allocate column ranges"));
         MGCT_TRY(launch_column_table(g, l, 0));
         MGCT_TRY(launch_column_table_df(g, l, 0));
     }

@@ -289,10 +289,11 @@ struct EpiPlus {
     }
 };
 
-// Where element (jv, ju) of view i of a weighted sinogram lies.  In float32 on
-// separable geometries it is [view][u][v], since the back-projector reads down
-// the detector columns (and the projector's lanes are the rows), with SINO_PAD
-// zero rows before every column and after the last; otherwise [view][v][u].
+// Where element (jv, ju) of view i of a weighted sinogram lies.  In float32
+// and with no or little detector tilt it is [view][u][v], since the
+// back-projector reads down the detector columns (and the column projector's
+// lanes are the rows), with SINO_PAD zero rows before every column and after
+// the last; otherwise [view][v][u].
 struct SinoStrides {
     int u, v;
     size_t view, first;
@@ -300,7 +301,9 @@ struct SinoStrides {
         return first + (size_t)i * view + (size_t)jv * v + (size_t)ju * u;
     }
 };
-inline bool columns_padded(const mgct_geom *g, size_t elem) { return g->separable && elem != 2; }
+inline bool columns_padded(const mgct_geom *g, size_t elem) {
+    return (g->separable || g->small_tilt) && elem != 2;
+}
 inline SinoStrides weighted_strides(const mgct_geom *g, const LevelInfo &L, size_t elem) {
     const int pitch = L.nv + SINO_PAD;
     return columns_padded(g, elem) ? SinoStrides{pitch, 1, (size_t)L.nu * pitch, SINO_PAD}

@@ -37,6 +37,13 @@ int launch_column_table_df(const mgct_geom *g, int level, cudaStream_t s) {
     return MGCT_OK;
 }
 
+int launch_class_ranges_tilt(const mgct_geom *g, int level, cudaStream_t s) {
+    const LevelInfo &L = g->lev[level];
+    const int K = g->desc.n_views;
+    MGCT_KERNEL(KK_OTHER, s, k_class_ranges_tilt<<<(K + 7) / 8, 256, 0, s>>>(L.d_views, K, L.nu, L.nv, L.d_ranges));
+    return MGCT_OK;
+}
+
 int launch_column_table(const mgct_geom *g, int level, cudaStream_t s) {
     const LevelInfo &L = g->lev[level];
     const int K = g->desc.n_views;
