@@ -15,10 +15,19 @@
 //   ds_u, ds_v: dS = one fine pixel along e_u / e_v;  dd_u, dd_v: dP likewise;
 //   psi: dP = u' Ev - v' Eu (the pixel offset turned about the normal).
 // The plane set and axis are held fixed (the integral is piecewise smooth).
+//
+// The march reads the projector's quad copies of the volume, one 16-byte load
+// a sample: bound by the issue of its ~45 operations.  Four tested loads from
+// the plain volume took 3.2 ms at 128^3 / 192^2 / 360 views, 2.2 ms with
+// the copies.
 #include "common.cuh"
 #include "project.cuh"
 
 namespace mgct {
+
+// Rays per n^2 from which the quad copies pay: they cost about 80 bytes a voxel
+// and save about 0.8 ps a sample, n samples a ray.
+constexpr double GG_QUAD_RAYS = 24.0;
 
 struct GradArgs {
     ProjArgs p;
@@ -26,9 +35,10 @@ struct GradArgs {
     double *part;    // [nviews][ublocks][5]
 };
 
-template <typename VT>
-__global__ void __launch_bounds__(PJ_BX *PJ_BY)
+template <typename VT>  // float: the plain volume and its transpose; float4: their quads
+__global__ void __launch_bounds__(PJ_BX *PJ_BY, 4)
     k_geom_grad(GradArgs ga, const VT *__restrict__ vol, const VT *__restrict__ volT) {
+    constexpr bool QUADS = std::is_same<VT, float4>::value;
     __shared__ ViewGeom G;
     __shared__ double red[5 * PJ_BX * PJ_BY / 32];
     const ProjArgs &a = ga.p;
@@ -39,6 +49,8 @@ __global__ void __launch_bounds__(PJ_BX *PJ_BY)
     __syncthreads();
     const int n = a.n;
     const float ic = 0.5f * (float)(n - 1);
+    const int side = quad_side(n);
+    const unsigned qmax = (unsigned)quad_elems(n) - 1u;
     const int ju = blockIdx.x * PJ_BX + threadIdx.x;
     double gsum[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     for (int v0 = 0; v0 < a.nv; v0 += PJ_BY) {
@@ -64,8 +76,10 @@ __global__ void __launch_bounds__(PJ_BX *PJ_BY)
         float lo = 0.0f, hi = (float)(n - 1);
         clip_planes(pb.hi, rb.hi, ic, (float)n, lo, hi);
         clip_planes(pz.hi, rz.hi, ic, (float)n, lo, hi);
-        const int i0 = max(0, (int)floorf(lo) - 1);
-        const int i1 = min(n - 1, (int)ceilf(hi) + 1);
+        // beyond these planes all four taps of a sample lie outside the volume,
+        // within them its corner lies in the quads (see ray_integral)
+        const int i0 = max(0, (int)floorf(lo));
+        const int i1 = lo <= hi ? min(n - 1, (int)ceilf(hi)) : -1;
         // t(i) = (i - S_a) / w_a
         const float rwa = 1.0f / wa.hi;
         const float Sa = G.S[ia];
@@ -84,14 +98,25 @@ __global__ void __launch_bounds__(PJ_BX *PJ_BY)
                 const float fb0 = floorf(gbk), fz0 = floorf(gzk);
                 const float tb = gbk - fb0, tz = gzk - fz0;
                 const int jb = Ib + (int)fb0, jz = Iz + (int)fz0;
-                const bool b0 = (unsigned)jb < (unsigned)n, b1 = (unsigned)(jb + 1) < (unsigned)n;
-                const bool z0 = (unsigned)jz < (unsigned)n, z1 = (unsigned)(jz + 1) < (unsigned)n;
-                const int row0 = (jz * n + pl) * n + jb;
-                const int row1 = row0 + n * n;
-                const float v00 = tap(base, row0, b0 && z0);
-                const float v10 = tap(base, row0 + 1, b1 && z0);
-                const float v01 = tap(base, row1, b0 && z1);
-                const float v11 = tap(base, row1 + 1, b1 && z1);
+                float v00, v10, v01, v11;
+                if constexpr (QUADS) {
+                    // the clip keeps q in range; the unsigned min only guarantees it
+                    const unsigned q = min((unsigned)(((jz + QD_PAD) * n + pl) * side + jb + QD_PAD), qmax);
+                    const float4 Q = __ldg(base + q);
+                    v00 = Q.x;
+                    v10 = Q.y;
+                    v01 = Q.z;
+                    v11 = Q.w;
+                } else {
+                    const bool b0 = (unsigned)jb < (unsigned)n, b1 = (unsigned)(jb + 1) < (unsigned)n;
+                    const bool z0 = (unsigned)jz < (unsigned)n, z1 = (unsigned)(jz + 1) < (unsigned)n;
+                    const int row0 = (jz * n + pl) * n + jb;
+                    const int row1 = row0 + n * n;
+                    v00 = tap(base, row0, b0 && z0);
+                    v10 = tap(base, row0 + 1, b1 && z0);
+                    v01 = tap(base, row1, b0 && z1);
+                    v11 = tap(base, row1 + 1, b1 && z1);
+                }
                 const float e0 = v10 - v00, e1 = v11 - v01;
                 const float a0 = fmaf(tb, e0, v00), a1 = fmaf(tb, e1, v01);
                 const float t = ((float)pl - Sa) * rwa;
@@ -175,7 +200,14 @@ extern "C" int mgct_geometry_grad(const mgct_geom *g, int level, int view0, int 
     ga.y = y;
     ga.part = g->d_scratch_part;
     dim3 grid(nub, nviews);
-    MGCT_KERNEL(KK_GEOMGRAD, s, k_geom_grad<float><<<grid, dim3(PJ_BX, PJ_BY), 0, s>>>(ga, vol, volT));
+    if ((double)nviews * L.nu * L.nv >= GG_QUAD_RAYS * (double)L.n * L.n) {
+        float4 *q1 = static_cast<float4 *>(g->d_scratch_quads), *q2 = q1 + quad_elems(L.n);
+        MGCT_TRY((launch_build_quads<float, float>(L.n, vol, q1, s)));
+        MGCT_TRY((launch_build_quads<float, float>(L.n, volT, q2, s)));
+        MGCT_KERNEL(KK_GEOMGRAD, s, k_geom_grad<float4><<<grid, dim3(PJ_BX, PJ_BY), 0, s>>>(ga, q1, q2));
+    } else {
+        MGCT_KERNEL(KK_GEOMGRAD, s, k_geom_grad<float><<<grid, dim3(PJ_BX, PJ_BY), 0, s>>>(ga, vol, volT));
+    }
     MGCT_KERNEL(KK_REDUCE, s, k_view_sums<<<(nviews + 127) / 128, 128, 0, s>>>(g->d_scratch_part, nub, nviews, dphi));
     return MGCT_OK;
 }
