@@ -334,15 +334,6 @@ struct PlaneTile {
 };
 
 // packed float pairs (one instruction each)
-__device__ __forceinline__ float2 add_f2(float2 a, float2 b) {
-    float2 d;
-    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
-        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
-        "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return d;
-}
 __device__ __forceinline__ float2 add_up_f2(float2 a, float2 b) {  // rounded toward plus infinity
     float2 d;
     asm("{\n\t.reg .b64 ra, rb, rd;\n\t"

@@ -293,15 +293,15 @@ __host__ __device__ inline size_t quad_elems(int n) { return (size_t)quad_side(n
 // packed 16-bit pairs for bf16 / fp16) [z + QD_PAD][i][b + QD_PAD]
 template <typename T, typename SRC = float>
 int launch_build_quads(int n, const SRC *src, void *dst, cudaStream_t s);
-// z-fastest quad copies for the column projector: src [z][i][b] ->
-// dst[i][b + QD_PAD][z + QD_PAD], each entry the footprint as two z pairs
+// z-fastest quad copies of v [z][y][x] for the column projector, of y-major
+// rays into zy (plane i = y, b = x) and of x-major rays into zx (i = x, b = y):
+// entry [i][b + QD_PAD][z + QD_PAD] holds the footprint as two z pairs
 // (V(jz, jb), V(jz + 1, jb)), (V(jz, jb + 1), V(jz + 1, jb + 1))
 template <typename T, typename SRC = float>
-int launch_build_zquads(int n, const SRC *src, void *dst, cudaStream_t s);
-// float32 z-fastest pairs for the column projector: (V(jz, jb), V(jz, jb + 1))
-// at dst[i][jb + QD_PAD][jz + QD_PAD], zero outside the volume
+int launch_build_zquads(int n, const SRC *v, void *zy, void *zx, cudaStream_t s);
+// float32 z-fastest pairs, likewise: (V(jz, jb), V(jz, jb + 1))
 template <typename SRC = float>
-int launch_build_zpairs(int n, const SRC *src, void *dst, cudaStream_t s);
+int launch_build_zpairs(int n, const SRC *v, void *zy, void *zx, cudaStream_t s);
 template <typename T>
 int launch_transpose_xy(int n, const T *in, T *out, cudaStream_t s);
 

@@ -232,10 +232,11 @@ __device__ __forceinline__ RaySum ray_integral(const ViewGeom &G, const ProjArgs
     return RaySum{acc, dl_h * a.h};
 }
 
-// Epilogue interface: operator()(i_batch, k_view, jv, ju, active, acc, dlh)
-// with A vol = acc * dlh at that ray, called by every thread of the block
-// (block reductions inside).  "Weighted" sinograms carry the factor dlh of
-// their ray, which the back-projector then need not recompute.
+// Epilogue interface: ray(i_batch, k_view, jv, ju, acc, dlh, s) with A vol =
+// acc * dlh at that ray, once per ray, adds its NV values to the thread's sums
+// s; finish(s) reduces them over the block (called by every thread).
+// "Weighted" sinograms carry the factor dlh of their ray, which the
+// back-projector then need not recompute.
 // Block order.  Consecutive views of the trajectory have nearby source
 // heights, and one detector-row tile of nearby views meets only a z-band of
 // the volume, so blocks are ordered (group of PJ_VG views, row tile, view in
@@ -262,8 +263,12 @@ __global__ void __launch_bounds__(PJ_BX *PJ_BY, MGCT_PJ_MINB)
     const int jv = vt * PJ_BY + threadIdx.y;
     const bool active = view_ok && ju < a.nu && jv < a.nv;
     RaySum rs{0.0f, 0.0f};
-    if (active) rs = ray_integral<VT>(G, a, ju, jv, vol, volT);
-    epi(i, k, jv, ju, active, rs.acc, rs.dlh);
+    double sums[2] = {0.0, 0.0};
+    if (active) {
+        rs = ray_integral<VT>(G, a, ju, jv, vol, volT);
+        epi.ray(i, k, jv, ju, rs.acc, rs.dlh, sums);
+    }
+    epi.finish(sums);
 }
 
 // out = A vol
@@ -271,9 +276,10 @@ template <typename OT>
 struct EpiStore {
     OT *out;
     int nu, nv;
-    __device__ void operator()(int i, int, int jv, int ju, bool active, float acc, float dlh) const {
-        if (active) out[((size_t)i * nv + jv) * nu + ju] = from_f32<OT>(acc * dlh);
+    __device__ void ray(int i, int, int jv, int ju, float acc, float dlh, double (&)[2]) const {
+        out[((size_t)i * nv + jv) * nu + ju] = from_f32<OT>(acc * dlh);
     }
+    __device__ void finish(double (&)[2]) const {}
 };
 
 // out = b + A vol (out may alias b: each ray reads its own entry first)
@@ -281,12 +287,11 @@ struct EpiPlus {
     float *out;
     const float *b;
     int nu, nv;
-    __device__ void operator()(int i, int, int jv, int ju, bool active, float acc, float dlh) const {
-        if (active) {
-            const size_t idx = ((size_t)i * nv + jv) * nu + ju;
-            out[idx] = b[idx] + acc * dlh;
-        }
+    __device__ void ray(int i, int, int jv, int ju, float acc, float dlh, double (&)[2]) const {
+        const size_t idx = ((size_t)i * nv + jv) * nu + ju;
+        out[idx] = b[idx] + acc * dlh;
     }
+    __device__ void finish(double (&)[2]) const {}
 };
 
 // Where element (jv, ju) of view i of a weighted sinogram lies.  In float32
@@ -321,25 +326,25 @@ struct EpiResidual {
     double *part;    // NULL: no norm
     int nu, nv, nviews;
     SinoStrides ws;
-    __device__ void operator()(int i, int, int jv, int ju, bool active, float acc, float dlh) const {
-        double s[1] = {0.0};
-        if (active) {
-            size_t idx = ((size_t)i * nv + jv) * nu + ju;
-            float r = __ldg(b + idx) - acc * dlh;
-            if (WEIGHTED) {
-                out[ws.at(i, jv, ju)] = from_f32<OT>(r * dlh);
-                s[0] = (double)r * (double)r;
-            } else {
-                OT ro = from_f32<OT>(r);
-                out[idx] = ro;
-                float rf = to_f32(ro);
-                s[0] = (double)rf * (double)rf;
-            }
+    __device__ void ray(int i, int, int jv, int ju, float acc, float dlh, double (&s)[2]) const {
+        size_t idx = ((size_t)i * nv + jv) * nu + ju;
+        float r = __ldg(b + idx) - acc * dlh;
+        if (WEIGHTED) {
+            out[ws.at(i, jv, ju)] = from_f32<OT>(r * dlh);
+            s[0] += (double)r * (double)r;
+        } else {
+            OT ro = from_f32<OT>(r);
+            out[idx] = ro;
+            float rf = to_f32(ro);
+            s[0] += (double)rf * (double)rf;
         }
+    }
+    __device__ void finish(double (&s)[2]) const {
         if (part) {
             __shared__ double red[PJ_BX * PJ_BY / 32];
-            block_sum<1>(s, red);
-            if (threadIdx.x == 0 && threadIdx.y == 0) part[block_linear()] = s[0];
+            double v[1] = {s[0]};
+            block_sum<1>(v, red);
+            if (threadIdx.x == 0 && threadIdx.y == 0) part[block_linear()] = v[0];
         }
     }
 };
@@ -353,14 +358,13 @@ struct EpiDualDot {
     double *part;  // [blocks][2]
     int nu, nv, nviews;
     SinoStrides ws;
-    __device__ void operator()(int i, int, int jv, int ju, bool active, float acc, float dlh) const {
-        double s[2] = {0.0, 0.0};
-        if (active) {
-            float rv = to_f32(rw[ws.at(i, jv, ju)]);
-            float ad = acc * dlh;
-            s[0] = (double)rv * (double)acc;
-            s[1] = (double)ad * (double)ad;
-        }
+    __device__ void ray(int i, int, int jv, int ju, float acc, float dlh, double (&s)[2]) const {
+        float rv = to_f32(rw[ws.at(i, jv, ju)]);
+        float ad = acc * dlh;
+        s[0] += (double)rv * (double)acc;
+        s[1] += (double)ad * (double)ad;
+    }
+    __device__ void finish(double (&s)[2]) const {
         __shared__ double red[2 * PJ_BX * PJ_BY / 32];
         block_sum<2>(s, red);
         if (threadIdx.x == 0 && threadIdx.y == 0) {
@@ -381,8 +385,7 @@ struct EpiEMTerms {
     const float *pi;
     int nu, nv, nviews;
     SinoStrides ws;
-    __device__ void operator()(int i, int k, int jv, int ju, bool active, float acc, float dlh) const {
-        if (!active) return;
+    __device__ void ray(int i, int k, int jv, int ju, float acc, float dlh, double (&)[2]) const {
         size_t pix = (size_t)jv * nu + ju;
         size_t full = (size_t)k * nv * nu + pix;
         float t = expf(-acc * dlh);
@@ -391,6 +394,7 @@ struct EpiEMTerms {
         o.y = t * __ldg(pi + full) * dlh;
         c[ws.at(i, jv, ju)] = o;
     }
+    __device__ void finish(double (&)[2]) const {}
 };
 
 // ---------------------------------------------------------------------------
@@ -437,7 +441,7 @@ __device__ __forceinline__ float2 quad_pair<float4>(const float4 &Q, int which) 
     return which ? make_float2(Q.z, Q.w) : make_float2(Q.x, Q.y);
 }
 
-// d = a * b + c and d = a - b on float pairs (one packed instruction each)
+// a * b + c, a + b and a - b on float pairs (one packed instruction each)
 __device__ __forceinline__ float2 fma_f2(float2 a, float2 b, float2 c) {
     float2 d;
     asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\t"
@@ -445,6 +449,15 @@ __device__ __forceinline__ float2 fma_f2(float2 a, float2 b, float2 c) {
         "fma.rn.f32x2 rd, ra, rb, rc;\n\tmov.b64 {%0, %1}, rd;\n\t}"
         : "=f"(d.x), "=f"(d.y)
         : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__device__ __forceinline__ float2 add_f2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
     return d;
 }
 __device__ __forceinline__ float2 sub_f2(float2 a, float2 b) {
@@ -627,7 +640,9 @@ __global__ void __launch_bounds__(PC_COLS *PC_ROWS, MGCT_PC_MINB)
     if (view_ok && ju < a.nu)  // uniform over the warp
         rs = column_rays<VT, LAYOUT>(a, cols + (size_t)k * 4 * a.nu + ju, jv, jv < a.nv, zqy, zqx,
                                      tab[threadIdx.y]);
-    epi(i, k, jv, ju, active, rs.acc, rs.dlh);
+    double sums[2] = {0.0, 0.0};
+    if (active) epi.ray(i, k, jv, ju, rs.acc, rs.dlh, sums);
+    epi.finish(sums);
 }
 
 template <typename VT, int LAYOUT, typename Epi>
@@ -684,9 +699,10 @@ int launch_project(const mgct_geom *g, int level, int view0, int nviews, int str
 }
 
 // A over views [view0, view0 + nviews * stride) of volume v (type SRC), read
-// through quad copies of storage type ST: the transpose of v into vT, the
-// quads of both ray classes into `quads` (2 quad_elems(n) entries), then the
-// column projector (tilt-free geometries) or k_project with epilogue `e`.
+// through copies of storage type ST in `quads` (room for 2 quad_elems(n)
+// entries): on tilt-free geometries pairs or quads of both ray classes and the
+// column projector; otherwise the transpose of v into vT, the quads of both
+// and k_project; with epilogue `e`.
 template <typename ST, typename SRC, typename Epi>
 int project_volume(const mgct_geom *g, int level, int view0, int nviews, int stride, const SRC *v, SRC *vT,
                    void *quads, const Epi &e, cudaStream_t s, int *nb) {
@@ -694,20 +710,18 @@ int project_volume(const mgct_geom *g, int level, int view0, int nviews, int str
     const LevelInfo &L = g->lev[level];
     QE *q1 = static_cast<QE *>(quads);
     QE *q2 = q1 + quad_elems(L.n);
-    MGCT_TRY(launch_transpose_xy<SRC>(L.n, v, vT, s));
     if (use_column_projector(g, level)) {
         if constexpr (std::is_same<ST, float>::value) {
             float2 *z1 = static_cast<float2 *>(quads);
             float2 *z2 = z1 + quad_elems(L.n);
-            MGCT_TRY((launch_build_zpairs<SRC>(L.n, v, z1, s)));
-            MGCT_TRY((launch_build_zpairs<SRC>(L.n, vT, z2, s)));
+            MGCT_TRY((launch_build_zpairs<SRC>(L.n, v, z1, z2, s)));
             return launch_project_col<Quad<ST>, ZL_PAIR>(g, level, view0, nviews, stride, z1, z2, e, s, nb);
         } else {
-            MGCT_TRY((launch_build_zquads<ST, SRC>(L.n, v, q1, s)));
-            MGCT_TRY((launch_build_zquads<ST, SRC>(L.n, vT, q2, s)));
+            MGCT_TRY((launch_build_zquads<ST, SRC>(L.n, v, q1, q2, s)));
             return launch_project_col<Quad<ST>, ZL_QUAD>(g, level, view0, nviews, stride, q1, q2, e, s, nb);
         }
     }
+    MGCT_TRY(launch_transpose_xy<SRC>(L.n, v, vT, s));
     MGCT_TRY((launch_build_quads<ST, SRC>(L.n, v, q1, s)));
     MGCT_TRY((launch_build_quads<ST, SRC>(L.n, vT, q2, s)));
     return launch_project<Quad<ST>>(g, level, view0, nviews, stride, q1, q2, e, s, nb);

@@ -301,13 +301,20 @@ static int osemtr(const mgct_geom *g, int level, int M, float *mu, const float *
     for (int m = 0; m < M; ++m) {
         int cnt = (K - m + M - 1) / M;
         if (cnt <= 0) continue;
-        MGCT_TRY(launch_transpose_xy<float>(L.n, mu, w.muT, s));
         EpiEMTerms e{w.c2, b, pi, L.nu, L.nv, cnt, weighted_strides(g, L, sizeof(float2))};
-        MGCT_TRY(launch_project<float>(g, level, m, cnt, M, mu, w.muT, e, s));
-        // c2 holds room for every view; past the largest subset's views it is free
-        const size_t all = padded_sino_elems(K, L.nu, L.nv), used = padded_sino_elems((K + M - 1) / M, L.nu, L.nv);
+        // c2 holds room for every view; past the largest subset's views it is
+        // free: room for the column projector's pairs, then for partial volumes
+        const size_t all = padded_sino_elems(K, L.nu, L.nv), used = (padded_sino_elems((K + M - 1) / M, L.nu, L.nv) + 1) & ~(size_t)1;
+        if (use_column_projector(g, level) && all >= used + 2 * quad_elems(L.n)) {
+            int nb = 0;
+            MGCT_TRY((project_volume<float, float>(g, level, m, cnt, M, mu, w.muT, w.c2 + used, e, s, &nb)));
+        } else {
+            MGCT_TRY(launch_transpose_xy<float>(L.n, mu, w.muT, s));
+            MGCT_TRY(launch_project<float>(g, level, m, cnt, M, mu, w.muT, e, s));
+        }
         MGCT_TRY(launch_backproject<2, float2, true>(g, level, m, cnt, M, w.c2, w.nd, 0, s,
-                                                     reinterpret_cast<float *>(w.c2 + used), 2 * (all - used)));
+                                                     reinterpret_cast<float *>(w.c2 + used),
+                                                     all > used ? 2 * (all - used) : 0));
         MGCT_TRY(launch_em_update(nv3, mu, w.nd, w.part, s));
     }
     return MGCT_OK;
