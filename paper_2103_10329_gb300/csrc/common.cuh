@@ -302,6 +302,9 @@ int launch_build_zquads(int n, const SRC *v, void *zy, void *zx, cudaStream_t s)
 // float32 z-fastest pairs, likewise: (V(jz, jb), V(jz, jb + 1))
 template <typename SRC = float>
 int launch_build_zpairs(int n, const SRC *v, void *zy, void *zx, cudaStream_t s);
+// z-fastest lines for the line projector, z padded with zeros to a multiple of
+// 4: v [z][y][x] -> ly [y][x][z] (y-major rays) and lx [x][y][z]
+int launch_build_lines(int n, const float *v, float *ly, float *lx, cudaStream_t s);
 template <typename T>
 int launch_transpose_xy(int n, const T *in, T *out, cudaStream_t s);
 

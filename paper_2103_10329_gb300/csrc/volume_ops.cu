@@ -161,6 +161,36 @@ int launch_build_zpairs(int n, const SRC *v, void *zy, void *zx, cudaStream_t s)
 }
 template int launch_build_zpairs<float>(int, const float *, void *, void *, cudaStream_t);
 
+// The line projector's copies: a 32 x 32 (z, x) tile of one y through shared
+// memory, read along x once, written along z into both (4 bytes read and 8
+// written a voxel; the transpose and two pair copies before moved 32).
+__global__ void __launch_bounds__(256) k_build_lines(int n, int pitch, const float *__restrict__ v,
+                                                     float *__restrict__ ly, float *__restrict__ lx) {
+    __shared__ float tile[32][33];
+    const int z0 = blockIdx.x * 32, x0 = blockIdx.y * 32, y = blockIdx.z;
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    for (int r = ty; r < 32; r += 8)
+        tile[r][tx] = z0 + r < n && x0 + tx < n ? __ldg(v + ((size_t)(z0 + r) * n + y) * n + x0 + tx) : 0.0f;
+    __syncthreads();
+    if (z0 + tx >= pitch) return;
+    const size_t plane = (size_t)(n + 2) * pitch;  // lines b = -1 .. n, the outer two zero
+    for (int r = ty; r < 32 && x0 + r < n; r += 8) {
+        const float w = tile[tx][r];
+        const int x = x0 + r;
+        ly[y * plane + (size_t)(x + 1) * pitch + z0 + tx] = w;
+        lx[x * plane + (size_t)(y + 1) * pitch + z0 + tx] = w;
+        if (x == 0) ly[y * plane + z0 + tx] = ly[y * plane + (size_t)(n + 1) * pitch + z0 + tx] = 0.0f;
+        if (y == 0) lx[x * plane + z0 + tx] = lx[x * plane + (size_t)(n + 1) * pitch + z0 + tx] = 0.0f;
+    }
+}
+
+int launch_build_lines(int n, const float *v, float *ly, float *lx, cudaStream_t s) {
+    const int pitch = ((n + 3) & ~3) + 4;  // line_pitch
+    dim3 grid((pitch + 31) / 32, (n + 31) / 32, n);
+    MGCT_KERNEL(KK_TRANSPOSE, s, k_build_lines<<<grid, dim3(32, 8), 0, s>>>(n, pitch, v, ly, lx));
+    return MGCT_OK;
+}
+
 // ---------------------------------------------------------------------------
 // Eq. 5 stencil: out = p * in, zero padding.  Block = 32 x 8 columns; each
 // thread walks ZB planes along z with three rolling halo planes in shared
@@ -244,7 +274,7 @@ static Stencil27 eq5_stencil(int slice_axis) {
 // (a float4 per thread and row, the x neighbours by lane shuffles), and a, b
 // roll in registers.  Every input element is read from HBM about once.
 // ---------------------------------------------------------------------------
-constexpr int PZ_TX = 128, PZ_TY = 8, PZ_ZB = 32, PZ_ST = 4, PZ_W = 136;  // slot row: x0-1 at column 3
+constexpr int PZ_TX = 128, PZ_TY = 8, PZ_ST = 4, PZ_W = 136;  // slot row: x0-1 at column 3
 
 __device__ __forceinline__ uint32_t sh_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void cpa4(float *dst, const float *src, bool valid) {
@@ -256,6 +286,7 @@ __device__ __forceinline__ void cpa16(float *dst, const float *src, int bytes) {
 }
 __device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 
+template <int PZ_ZB>
 __global__ void __launch_bounds__(PZ_TX / 4 * PZ_TY) k_precondition_z(int n, const float *__restrict__ in,
                                                                       float *__restrict__ out) {
     __shared__ __align__(16) float pl[PZ_ST][PZ_TY + 2][PZ_W];
@@ -361,8 +392,16 @@ int launch_precondition(int n, int slice_axis, const float *in, float *out, cuda
         return MGCT_OK;
     }
     if (slice_axis == 2) {
-        dim3 grid((n + PZ_TX - 1) / PZ_TX, (n + PZ_TY - 1) / PZ_TY, (n + PZ_ZB - 1) / PZ_ZB);
-        MGCT_KERNEL(KK_PRECONDITION, s, k_precondition_z<<<grid, PZ_TX / 4 * PZ_TY, 0, s>>>(n, in, out));
+        // 32 planes a block where that fills the chip; 8, with a halo of a quarter
+        // instead of a sixteenth, where each block's walk along z is what takes
+        // the time (64^3: 16 blocks, 24 us a launch; 64 blocks, 10 us)
+        dim3 grid((n + PZ_TX - 1) / PZ_TX, (n + PZ_TY - 1) / PZ_TY, (n + 31) / 32);
+        if (n > 160) {
+            MGCT_KERNEL(KK_PRECONDITION, s, k_precondition_z<32><<<grid, PZ_TX / 4 * PZ_TY, 0, s>>>(n, in, out));
+        } else {
+            grid.z = (n + 7) / 8;
+            MGCT_KERNEL(KK_PRECONDITION, s, k_precondition_z<8><<<grid, PZ_TX / 4 * PZ_TY, 0, s>>>(n, in, out));
+        }
         return MGCT_OK;
     }
     dim3 grid((n + ST_BX - 1) / ST_BX, (n + ST_BY - 1) / ST_BY, (n + ST_ZB - 1) / ST_ZB);
@@ -601,18 +640,22 @@ int launch_bilateral(int n, const float *in, float *out, double sigma_s, double 
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(1024) k_sum_partials(const double *__restrict__ part, int count, int nvals,
                                                        double *__restrict__ out) {
-    __shared__ double red[1024];
+    __shared__ double red[2][32];
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+    double s[2] = {0.0, 0.0};
+    for (int i = threadIdx.x; i < count; i += 1024)
+        for (int c = 0; c < nvals; ++c) s[c] += part[(size_t)i * nvals + c];
     for (int c = 0; c < nvals; ++c) {
-        double s = 0.0;
-        for (int i = threadIdx.x; i < count; i += 1024) s += part[(size_t)i * nvals + c];
-        red[threadIdx.x] = s;
-        __syncthreads();
-        for (int w = 512; w > 0; w >>= 1) {
-            if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) out[c] = red[0];
-        __syncthreads();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s[c] += __shfl_down_sync(0xffffffffu, s[c], o);
+        if (lane == 0) red[c][warp] = s[c];
+    }
+    __syncthreads();
+    if (warp < nvals) {
+        double t = red[warp][lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+        if (lane == 0) out[warp] = t;
     }
 }
 
