@@ -76,9 +76,13 @@ __global__ void __launch_bounds__(PJ_BX *PJ_BY, 4)
         float lo = 0.0f, hi = (float)(n - 1);
         clip_planes(pb.hi, rb.hi, ic, (float)n, lo, hi);
         clip_planes(pz.hi, rz.hi, ic, (float)n, lo, hi);
-        // beyond these planes all four taps of a sample lie outside the volume,
-        // within them its corner lies in the quads (see ray_integral)
-        const int i0 = max(0, (int)floorf(lo));
+        // a plane before the first with a tap in the volume, up to the last: a
+        // sample moves by at most a voxel a plane, so its corner lies in
+        // [-QD_PAD, n + 1], the quads' range, and the first adds zeros.  dB/df
+        // jumps at the voxel centres, so the crossings' rounding, which the
+        // first chunk's anchor sets, is part of the result: starting a plane
+        // later changed the gradient by 3e-4 at 128^3.
+        const int i0 = max(0, (int)floorf(lo) - 1);
         const int i1 = lo <= hi ? min(n - 1, (int)ceilf(hi)) : -1;
         // t(i) = (i - S_a) / w_a
         const float rwa = 1.0f / wa.hi;
@@ -100,7 +104,7 @@ __global__ void __launch_bounds__(PJ_BX *PJ_BY, 4)
                 const int jb = Ib + (int)fb0, jz = Iz + (int)fz0;
                 float v00, v10, v01, v11;
                 if constexpr (QUADS) {
-                    // the clip keeps q in range; the unsigned min only guarantees it
+                    // q is in range (see above); the unsigned min only guarantees it
                     const unsigned q = min((unsigned)(((jz + QD_PAD) * n + pl) * side + jb + QD_PAD), qmax);
                     const float4 Q = __ldg(base + q);
                     v00 = Q.x;
