@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "conv3d_out.cuh"
 #include "conv3d_tc.cuh"
 
 namespace mgct {
@@ -509,9 +510,10 @@ int mgct_net_create(uint64_t seed, mgct_net **out) {
 // `normalise`, x is divided by its RMS (computed here).  Leaves the
 // activations in the workspace.
 // ss: device sum of squares of the whole volume (x is scaled by 1 / RMS with
-// RMS = sqrt(ss / nnorm)), or NULL for no scaling.
+// RMS = sqrt(ss / nnorm)), or NULL for no scaling.  inference: the output
+// layer by k_conv_out where its grid allows (conv3d_out.cuh).
 static int net_forward(const mgct_net *net, int B, int D, int H, int W, const float *x, const double *ss,
-                       double nnorm, const NetSpace &sp, cudaStream_t s) {
+                       double nnorm, const NetSpace &sp, bool inference, cudaStream_t s) {
     const int nvox = B * D * H * W;
     MGCT_KERNEL(KK_CONV, s, k_net_input<<<std::min((nvox + 255) / 256, 152 * 32), 256, 0, s>>>(x, ss, nnorm, nvox, sp.x0, sp.xs));
     const __nv_bfloat16 *cur = sp.x0;
@@ -526,6 +528,10 @@ static int net_forward(const mgct_net *net, int B, int D, int H, int W, const fl
         a.H = H;
         a.W = W;
         a.nvox = nvox;
+        if (inference && l == NL - 1 && conv_out_fits(B, D, H, W)) {
+            MGCT_TRY(launch_conv_out(cur, net->wf[l], LCOUT[l], net->b[l], sp.y, B, D, H, W, s));
+            break;
+        }
         if (l < NL - 1) {
             a.out = sp.act[l];
             a.out_ch = LCOUT[l];
@@ -583,7 +589,7 @@ int mgct_net_apply(const mgct_net *net, int B, int D, int H, int W, const float 
     if (ws_bytes >= mgct_net_workspace_bytes(nvox, 0)) {
         carve_net(nvox, false, static_cast<char *>(ws), &sp);
         MGCT_TRY(net_sumsq(dir, (int)nvox, sp.sumsq, sp.lpart, s));
-        MGCT_TRY(net_forward(net, B, D, H, W, dir, sp.sumsq, (double)nvox, sp, s));
+        MGCT_TRY(net_forward(net, B, D, H, W, dir, sp.sumsq, (double)nvox, sp, true, s));
         MGCT_KERNEL(KK_CONV, s, k_net_output<<<std::min((int)((nvox + 255) / 256), 152 * 32), 256, 0, s>>>(
                                     sp.xs, sp.y, sp.sumsq, (double)nvox, (int)nvox, net->err, out));
         return MGCT_OK;
@@ -605,7 +611,7 @@ int mgct_net_apply(const mgct_net *net, int B, int D, int H, int W, const float 
             const int z1 = std::min(D, z0 + S);
             const int zs = std::max(0, z0 - NET_HALO), ze = std::min(D, z1 + NET_HALO);
             const int64_t base = ((int64_t)b * D + zs) * plane;
-            MGCT_TRY(net_forward(net, 1, ze - zs, H, W, dir + base, sp.sumsq, (double)nvox, sp, s));
+            MGCT_TRY(net_forward(net, 1, ze - zs, H, W, dir + base, sp.sumsq, (double)nvox, sp, true, s));
             const int64_t off = (int64_t)(z0 - zs) * plane, cnt = (int64_t)(z1 - z0) * plane;
             MGCT_KERNEL(KK_CONV, s, k_net_output<<<std::min((int)((cnt + 255) / 256), 152 * 32), 256, 0, s>>>(
                                         sp.xs + off, sp.y + off, sp.sumsq, (double)nvox, (int)cnt, net->err,
@@ -630,7 +636,7 @@ int mgct_net_forward_backward(mgct_net *net, int B, int D, int H, int W, const f
     carve_net(nvox, true, static_cast<char *>(ws), &sp);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     // x and t are already in scaled units
-    MGCT_TRY(net_forward(net, B, D, H, W, x, nullptr, 1.0, sp, s));
+    MGCT_TRY(net_forward(net, B, D, H, W, x, nullptr, 1.0, sp, false, s));
     const int nb = std::min(1024, (nvox + 255) / 256);
     MGCT_KERNEL(KK_CONV, s, k_mse<<<nb, 256, 0, s>>>(sp.xs, sp.y, t, nvox, net->err, sp.g[NL - 1], sp.lpart));
     MGCT_TRY(launch_sum_partials(sp.lpart, nb, 1, net->loss, s));
