@@ -1013,7 +1013,7 @@ def evaluation_1024(args):
 
 def family_rooflines(W, nnz, trace0, peaks, sm_clock, fp32_peak, mp=None):
     """Roofline objects of the projector and back-projector families on the
-    finest grid: one grid-0 launch is one A (or A^T) over every view.  The
+    finest grid: one grid-0 "launch" is one A (or A^T: two launches) over every view.  The
     fraction is t_floor / t_launch with t_floor the largest of three floors
     per launch:
       HBM: one volume plus one sinogram at the measured copy bandwidth;
@@ -1031,12 +1031,14 @@ def family_rooflines(W, nnz, trace0, peaks, sm_clock, fp32_peak, mp=None):
     floors = {"hbm_ms": hbm_b / (peaks.get("hbm_gbs", 6790.0) * 1e9) * 1e3,
               "onchip_gather_ms": gather_b / l1_peak * 1e3,
               "fp32_ms": fl / (fp32_peak * 1e12) * 1e3}
-    names = {"project": "k_project_col", "backproject": "k_backproject_reg"}
+    names = {"project": "k_project_lines" if n >= 448 else "k_project_col", "backproject": "k_backproject_plane"}
     out = {}
     for fam, kname in names.items():
         if fam not in trace0 or not trace0[fam][1]:
             continue
         t0_ms, t0_n = trace0[fam]
+        if fam == "backproject":
+            t0_n //= 2  # an A^T: both ray classes and the sum of their partial volumes, or a launch per class
         avg_ms = t0_ms / max(t0_n, 1)
         t_s = avg_ms / 1e3
         tr = traffic_record(kname)

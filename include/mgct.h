@@ -146,9 +146,9 @@ int mgct_project(const mgct_geom *geom, int level, int view0, int nviews, int vi
  * The exact transpose of mgct_project's weights: for each voxel and view,
  * every detector pixel whose ray crosses the voxel's plane (along that ray's
  * major axis) within one voxel of it contributes
- * y * h_g|w|/|w_a| * hat(db) * hat(dc).  On tilt-free geometries each ray's
- * y * h_g|w|/|w_a| is formed in the handle's quad scratch (in chunks of
- * views) and splatted by z-slab into shared memory; with detector tilt, or a
+ * y * h_g|w|/|w_a| * hat(db) * hat(dc).  Each ray's y * h_g|w|/|w_a| is formed
+ * in the handle's quad scratch (in chunks of views) and back-projected plane
+ * by plane; with the detector turned by more than 0.35 from upright, or a
  * scratch smaller than one view, a per-voxel gather computes the same sums.
  * No atomics: the result is deterministic.  sino: batch sinogram of dtype
  * st; vol_out: float32 [n_g]^3, overwritten (accumulate = 0) or added to
