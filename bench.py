@@ -1129,6 +1129,31 @@ def time_steps(rec, vol, steps, warmup, barrier=lambda: None, clocks=None):
     return ms, launches, trace, trace0, clk
 
 
+def headline(full):
+    """The JSON line: `full` without its long parts (25 KB with them, which a
+    reader of the end of the output does not see whole), each replaced by its
+    summary.  The whole of it goes to stderr."""
+    line = {k: v for k, v in full.items()
+            if k not in ("roofline", "rooflines", "kernels", "secondary", "hbm_kernels", "time_to_accuracy",
+                         "joint_drift_estimation", "oracle_beside")}
+    keep = ("kernel", "bound", "achieved", "peak", "unit", "frac", "avg_launch_ms", "launches_timed", "traffic")
+    line["roofline"] = full["roofline"] and {k: full["roofline"].get(k) for k in keep}
+    if full.get("rooflines"):
+        line["rooflines"] = {f: {k: r.get(k) for k in ("kernel", "frac", "avg_launch_ms")}
+                             for f, r in full["rooflines"].items()}
+    if full.get("secondary"):
+        line["secondary"] = {k: full["secondary"][k] for k in ("config", "value", "unit", "ms_per_step")}
+    tta = full.get("time_to_accuracy")
+    if tta:
+        line["time_to_accuracy"] = {
+            "E2": tta.get("E2_pmgl_fp32_2iter"),
+            "ms_to_E2": {f: r.get("ms_to_E2") for f, r in (tta.get("forms") or {}).items()},
+            "seconds_to_rmse_1e-3": {w: {f: q.get("seconds") for f, q in (r.get("forms") or {}).items()}
+                                     for w, r in (tta.get("literal_rmse_1e-3") or {}).items()}}
+    line["details"] = "the whole record: one JSON line on stderr"
+    return line
+
+
 def gpu_arm(args, rank, world):
     import torch
     from paper_2103_10329_gb300 import build, mgct
@@ -1297,7 +1322,8 @@ def gpu_arm(args, rank, world):
                                                   "conflict-free 16-byte shared loads"},
                 "secondary": second, "hbm_kernels": hbm, "time_to_accuracy": tta, "joint_drift_estimation": joint_c4,
                 "oracle_beside": beside}
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(headline(line)), flush=True)
 
 
 def main():
