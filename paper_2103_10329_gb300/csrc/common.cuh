@@ -133,6 +133,7 @@ void trace_begin(int kind, cudaStream_t s);
 void trace_end(int kind, cudaStream_t s);
 void trace_tag(int tag);  // grid level of the launches that follow (this thread)
 int check_ptr(const void *p, const char *name, bool may_be_null = false);
+int sm_count(int *sms);  // multiprocessors of the current device
 
 #define MGCT_TRY(...)                   \
     do {                                \

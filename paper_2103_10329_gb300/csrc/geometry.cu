@@ -29,6 +29,12 @@ int check_cuda(cudaError_t e, const char *what) {
                      std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+int sm_count(int *sms) {
+    int dev = 0;
+    MGCT_TRY(check_cuda(cudaGetDevice(&dev), "device"));
+    return check_cuda(cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev), "device");
+}
+
 void count_launch(int n) { g_launches += (uint64_t)n; }
 
 int check_ptr(const void *p, const char *name, bool may_be_null) {

@@ -534,13 +534,18 @@ int launch_prolong_add(int nc, const float *cn, const float *co, float *fine, cu
 // Alg. 1 BilateralFilter: out(p) = sum_q w x(q) / sum_q w over the window
 // |q - p|_inf <= R inside the volume, w = exp(-|q - p|^2 / 2 ss^2 -
 // (x(q) - x(p))^2 / 2 sr^2): one base-2 exponential per neighbour, the self
-// weight is 1.  A block owns 32 x 8 columns over BL_ZB planes; planes with
+// weight is 1.  A block owns 32 x 8 columns over ZB planes; planes with
 // their halo pass through a ring of 2 R + 2 shared-memory slots, the next one
 // loaded while the current one is filtered, and a neighbour's place inside the
 // volume is tested only in blocks at the volume's faces.  Bound by the
 // exponentials (26 at R = 1: 0.72 ms per 512^3 volume at 16 a clock and SM)
 // and the issue of the six operations around each; the window read through L1
 // with every neighbour tested took 3.48 ms.
+//
+// A block walks 16 planes where that leaves two blocks for each multiprocessor, and
+// one in smaller volumes, whose time is one block's walk (radius 1 and 4, us, with
+// 16 planes and with 1: 24^3 29 and 8, 545 and 42; 64^3 27 and 8, 555 and 120; 96^3
+// 29 and 19, 628 and 452).
 // ---------------------------------------------------------------------------
 constexpr int BL_ZB = 16;
 
@@ -578,14 +583,14 @@ __device__ __forceinline__ float bilateral_at(const float (&pl)[2 * R + 2][8 + 2
     return num / den;
 }
 
-template <int R>
+template <int R, int ZB>
 __global__ void __launch_bounds__(256) k_bilateral(int n, const float *__restrict__ in, float *__restrict__ out,
                                                    float ks, float kr) {
     constexpr int S = 2 * R + 2, H = 8 + 2 * R, W = 32 + 2 * R, NL = (H * W + 255) / 256;
     __shared__ float pl[S][H][W];
     const int tid = threadIdx.x + 32 * threadIdx.y;
-    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 8, z0 = blockIdx.z * BL_ZB;
-    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, z1 = min(n, z0 + BL_ZB);
+    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 8, z0 = blockIdx.z * ZB;
+    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, z1 = min(n, z0 + ZB);
     const size_t nn = (size_t)n * n;
     float v[NL];
     auto fetch = [&](int z) {  // plane z into registers, 0 outside the volume
@@ -609,7 +614,7 @@ __global__ void __launch_bounds__(256) k_bilateral(int n, const float *__restric
         store(z);
     }
     __syncthreads();
-    const bool face = x0 < R || y0 < R || z0 < R || x0 + 32 + R > n || y0 + 8 + R > n || z0 + BL_ZB + R > n;
+    const bool face = x0 < R || y0 < R || z0 < R || x0 + 32 + R > n || y0 + 8 + R > n || z0 + ZB + R > n;
     for (int z = z0; z < z1; ++z) {
         fetch(z + R + 1);
         if (x < n && y < n) {
@@ -621,17 +626,30 @@ __global__ void __launch_bounds__(256) k_bilateral(int n, const float *__restric
     }
 }
 
+template <int R>
+int launch_bilateral_r(int n, const float *in, float *out, float ks, float kr, cudaStream_t s) {
+    int sms = 0;
+    MGCT_TRY(sm_count(&sms));
+    dim3 grid((n + 31) / 32, (n + 7) / 8, (n + BL_ZB - 1) / BL_ZB);
+    const dim3 block(32, 8);
+    if ((long long)grid.x * grid.y * grid.z >= 2LL * sms) {
+        MGCT_KERNEL(KK_UPDATE, s, k_bilateral<R, BL_ZB><<<grid, block, 0, s>>>(n, in, out, ks, kr));
+    } else {
+        grid.z = n;
+        MGCT_KERNEL(KK_UPDATE, s, k_bilateral<R, 1><<<grid, block, 0, s>>>(n, in, out, ks, kr));
+    }
+    return MGCT_OK;
+}
+
 int launch_bilateral(int n, const float *in, float *out, double sigma_s, double sigma_r, int radius, cudaStream_t s) {
-    dim3 grid((n + 31) / 32, (n + 7) / 8, (n + BL_ZB - 1) / BL_ZB), block(32, 8);
     const double log2e = 1.4426950408889634;
     const float ks = (float)(-0.5 * log2e / (sigma_s * sigma_s)), kr = (float)(-0.5 * log2e / (sigma_r * sigma_r));
     switch (radius) {
-        case 1: MGCT_KERNEL(KK_UPDATE, s, k_bilateral<1><<<grid, block, 0, s>>>(n, in, out, ks, kr)); break;
-        case 2: MGCT_KERNEL(KK_UPDATE, s, k_bilateral<2><<<grid, block, 0, s>>>(n, in, out, ks, kr)); break;
-        case 3: MGCT_KERNEL(KK_UPDATE, s, k_bilateral<3><<<grid, block, 0, s>>>(n, in, out, ks, kr)); break;
-        default: MGCT_KERNEL(KK_UPDATE, s, k_bilateral<4><<<grid, block, 0, s>>>(n, in, out, ks, kr)); break;
+        case 1: return launch_bilateral_r<1>(n, in, out, ks, kr, s);
+        case 2: return launch_bilateral_r<2>(n, in, out, ks, kr, s);
+        case 3: return launch_bilateral_r<3>(n, in, out, ks, kr, s);
+        default: return launch_bilateral_r<4>(n, in, out, ks, kr, s);
     }
-    return MGCT_OK;
 }
 
 // ---------------------------------------------------------------------------
