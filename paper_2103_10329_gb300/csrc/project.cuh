@@ -274,6 +274,7 @@ __global__ void __launch_bounds__(PJ_BX *PJ_BY, MGCT_PJ_MINB)
 // out = A vol
 template <typename OT>
 struct EpiStore {
+    static constexpr bool SMALL_BATCH = true;
     OT *out;
     int nu, nv;
     __device__ void ray(int i, int, int jv, int ju, float acc, float dlh, double (&)[2]) const {
@@ -284,6 +285,7 @@ struct EpiStore {
 
 // out = b + A vol (out may alias b: each ray reads its own entry first)
 struct EpiPlus {
+    static constexpr bool SMALL_BATCH = false;
     float *out;
     const float *b;
     int nu, nv;
@@ -321,6 +323,7 @@ inline SinoStrides weighted_strides(const mgct_geom *g, const LevelInfo &L, size
 // the strides ws.
 template <typename OT, bool WEIGHTED = false>
 struct EpiResidual {
+    static constexpr bool SMALL_BATCH = WEIGHTED;
     OT *out;
     const float *b;  // [i][v][u]
     double *part;    // NULL: no norm
@@ -354,6 +357,7 @@ struct EpiResidual {
 //   |A d|^2  = sum (acc * dlh)^2
 template <typename RT>
 struct EpiDualDot {
+    static constexpr bool SMALL_BATCH = true;
     const RT *rw;
     double *part;  // [blocks][2]
     int nu, nv, nviews;
@@ -380,6 +384,7 @@ struct EpiDualDot {
 // b and PI are full [K][nv][nu] arrays indexed by the view k; c is a batch
 // two-channel sinogram at the strides ws.
 struct EpiEMTerms {
+    static constexpr bool SMALL_BATCH = false;
     float2 *c;
     const float *b;
     const float *pi;
@@ -428,12 +433,16 @@ struct EpiEMTerms {
 // all-zero entry; planes past the union (the last batch) read the zero entry
 // row (plane 0, corner b = n + 1).  The clamp is exact, not a guard band.
 // ---------------------------------------------------------------------------
-// Plane loads in flight per ray, and resident blocks per SM: 8 and 4; pairs of
-// volumes up to PC_SMALL_N a side 4 and 6, where the copies stay in L2 whatever
-// runs beside (256^3 / 720 views 15.1 ms a projection against 15.5, 440^3 / 200
-// views 23.7 against 22.6: there more resident blocks spread over more of the
-// volume than L2 holds).
-constexpr int PC_BATCH = 8, PC_BATCH_SMALL = 4, PC_SMALL_N = 300;
+// Plane loads in flight per ray, and resident blocks per SM: 8 and 4, or 4 and 6
+// for pairs in launches of many views of volumes up to 300 a side, whose copies
+// L2 holds whatever runs beside.  Both projections of a Landweber step by views,
+// 8 loads and 4: 128^3 16 views 127 and 129 us, 48 337 and 322, 360 2290 and
+// 2163; 200^3 32 views 0.90 and 0.94 ms, 48 1.28 and 1.24; 256^3 64 views 3.27
+// and 3.39 ms, 128 6.05 and 6.00, 720 32.5 and 31.6; 300^3 128 views 10.7 and
+// 10.8, 240 19.4 and 19.1.  Epilogues that were not faster say so (SMALL_BATCH):
+// a plain residual of 256^3 / 60 views took 1.49 ms with 8 and 2.29 with 4.
+constexpr int PC_BATCH = 8, PC_BATCH_SMALL = 4;
+inline bool use_small_batch(int n, int nviews) { return n <= 300 && nviews >= 48 && (n <= 200 || nviews >= n); }
 constexpr int PC_TAB = 32;               // planes per table refill (one per lane)
 
 template <typename E>
@@ -663,8 +672,8 @@ int launch_project_col(const mgct_geom *g, int level, int view0, int nviews, int
     dim3 grid((L.nu + PC_COLS - 1) / PC_COLS, vg, groups * ((L.nv + PC_ROWS - 1) / PC_ROWS));
     if (nblocks) *nblocks = (int)project_blocks_col(L.nu, L.nv, nviews);
     if (nviews == 0) return MGCT_OK;
-    if constexpr (LAYOUT == ZL_PAIR) {
-        if (L.n <= PC_SMALL_N) {
+    if constexpr (LAYOUT == ZL_PAIR && Epi::SMALL_BATCH) {
+        if (use_small_batch(L.n, nviews)) {
             MGCT_KERNEL(KK_PROJECT, s, k_project_col<VT, LAYOUT, PC_BATCH_SMALL, Epi>
                                        <<<grid, dim3(PC_ROWS, PC_COLS), 0, s>>>(a, L.d_cols_df, zqy, zqx, epi));
             return MGCT_OK;
