@@ -25,9 +25,14 @@
 
 namespace mgct {
 
-// Rays per n^2 from which the quad copies pay: they cost about 80 bytes a voxel
-// and save about 0.8 ps a sample, n samples a ray.
-constexpr double GG_QUAD_RAYS = 24.0;
+// The quad copies pay from 24 rays per n^2 where both classes' fit L2 (up to
+// 160^3; with 24.75 n^2 rays, plain and quads: 64^3 0.20 and 0.18 ms, 128^3 0.71
+// and 0.64), from 50 beyond (256^3 with 25, 36, 54, 72 n^2: 3.2 and 3.4, 3.1 and
+// 3.6, 3.9 and 3.8, 4.2 and 3.8 ms), and never below 28^3, where their two
+// launches are longer than the march (24^3 49 and 53 us, 16^3 31 and 38).
+inline bool use_quads(int n, double rays) {
+    return n >= 28 && rays >= (n <= 160 ? 24.0 : 50.0) * n * n;
+}
 
 struct GradArgs {
     ProjArgs p;
@@ -76,9 +81,11 @@ __global__ void __launch_bounds__(PJ_BX *PJ_BY, 4)
         float lo = 0.0f, hi = (float)(n - 1);
         clip_planes(pb.hi, rb.hi, ic, (float)n, lo, hi);
         clip_planes(pz.hi, rz.hi, ic, (float)n, lo, hi);
-        // a plane before the first with a tap in the volume, up to the last: a
-        // sample moves by at most a voxel a plane, so its corner lies in
-        // [-QD_PAD, n + 1], the quads' range, and the first adds zeros.  dB/df
+        // from less than two planes before the crossings reach -1, where a tap
+        // in the volume can first have a weight, up to the last with one: a
+        // sample moves by at most a voxel a plane, so crossings stay above -3
+        // and below n + 1, corners in [-QD_PAD, n + 1], the quads' range, and
+        // the planes before the first with a tap add zeros.  dB/df
         // jumps at the voxel centres, so the crossings' rounding, which the
         // first chunk's anchor sets, is part of the result: starting a plane
         // later changed the gradient by 3e-4 at 128^3.
@@ -204,7 +211,7 @@ extern "C" int mgct_geometry_grad(const mgct_geom *g, int level, int view0, int 
     ga.y = y;
     ga.part = g->d_scratch_part;
     dim3 grid(nub, nviews);
-    if ((double)nviews * L.nu * L.nv >= GG_QUAD_RAYS * (double)L.n * L.n) {
+    if (use_quads(L.n, (double)nviews * L.nu * L.nv)) {
         float4 *q1 = static_cast<float4 *>(g->d_scratch_quads), *q2 = q1 + quad_elems(L.n);
         MGCT_TRY((launch_build_quads<float, float>(L.n, vol, q1, s)));
         MGCT_TRY((launch_build_quads<float, float>(L.n, volT, q2, s)));
