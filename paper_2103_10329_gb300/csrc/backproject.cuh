@@ -20,6 +20,9 @@
 // atomics.
 #pragma once
 
+#include <algorithm>
+#include <cmath>
+
 #include "common.cuh"
 #include "project.cuh"
 
@@ -1097,17 +1100,21 @@ __global__ void k_sum_parts(size_t len, int parts, const float *__restrict__ par
 
 namespace mgct {
 
-// Number of view shares for a tile-kernel launch of `blocks` tiles: the one
-// that fills whole waves of resident blocks best (a launch of 3.4 waves takes
-// as long as one of 4; coarse grids and OS-EMTR subsets fill a fraction of
-// one), at most 16 and `most`.  Each share beyond the first has to gain 4 %
-// for its partial volume and set-up.
-inline int plane_splits(int resident, int blocks, int nviews, int most) {
+// Number of view shares for a launch of `blocks` blocks on `sms` multiprocessors
+// that hold `occ` blocks each, at most 16 and `most`: the one with the least
+// estimated time, in units of a view's work on a full chip.  The multiprocessor
+// with the most blocks, m of them, takes m / occ waves, of which a last one of r
+// blocks takes 0.4 + 0.45 r / occ; every share writes and reads its partial
+// volumes, `share` views' work: 1.5 in the plane kernel at a row step of 0.6 voxel
+// (public call at 128^3 by 1, 2, 3 shares: 16 views 110, 100, 111 us, 90 views 493,
+// 397, 381; at 200^3, 4 views by 1, 2, 4: 125, 168, 256 us), 0.5 in the tilt kernel.
+inline int view_splits(int sms, int occ, int blocks, int nviews, int most, double share) {
     int best = 1;
     double cost = 1e300;
     for (int sp = 1; sp <= 16 && sp <= nviews && (sp == 1 || sp <= most); ++sp) {
-        const double waves = (double)(((long long)blocks * sp + resident - 1) / resident);
-        const double c = waves / sp * (1.0 + 0.04 * (sp - 1));
+        const long long m = ((long long)blocks * sp + sms - 1) / sms;
+        const double waves = (double)(m / occ) + (m % occ ? 0.4 + 0.45 * (double)(m % occ) / occ : 0.0);
+        const double c = nviews * waves * occ * sms / ((double)blocks * sp) + share * sp;
         if (c < cost) {
             cost = c;
             best = sp;
@@ -1121,18 +1128,17 @@ inline int plane_splits(int resident, int blocks, int nviews, int most) {
 // of split_buf (cap floats), or one class after the other without one.
 template <int NCH, typename F, typename KF>
 int launch_tiles(const LevelInfo &L, BPArgs a, dim3 grid, KF kernel, size_t smem, float *out, int accumulate,
-                 cudaStream_t s, float *split_buf, size_t cap, F run) {
+                 cudaStream_t s, float *split_buf, size_t cap, double share, F run) {
     const size_t vol_floats = (size_t)NCH * L.n * L.n * L.n;
     const int room = split_buf ? (int)(cap / vol_floats < 64 ? cap / vol_floats : 64) : 0;
     if (room < 2) {
         for (a.cls = 1; a.cls >= 0; --a.cls) MGCT_KERNEL(KK_BACKPROJECT, s, run(a, grid, out, accumulate || a.cls == 0));
         return MGCT_OK;
     }
-    int dev = 0, sms = 0, occ = 0;
-    MGCT_TRY(check_cuda(cudaGetDevice(&dev), "device"));
-    MGCT_TRY(check_cuda(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device"));
+    int sms = 0, occ = 0;
+    MGCT_TRY(sm_count(&sms));
     MGCT_TRY(check_cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, 32 * BT_WARPS, smem), "occupancy"));
-    a.splits = plane_splits(sms * (occ > 0 ? occ : 1), 2 * (int)(grid.x * grid.y * grid.z), a.nviews, room / 2);
+    a.splits = view_splits(sms, occ > 0 ? occ : 1, 2 * (int)(grid.x * grid.y * grid.z), a.nviews, room / 2, share);
     const int parts = 2 * a.splits;
     grid.z *= parts;
     MGCT_KERNEL(KK_BACKPROJECT, s, run(a, grid, split_buf, 0));
@@ -1143,12 +1149,14 @@ int launch_tiles(const LevelInfo &L, BPArgs a, dim3 grid, KF kernel, size_t smem
 
 template <int NCH, int NP, typename ST>
 int launch_backproject_plane(const LevelInfo &L, const BPArgs &a, const ST *sino, float *out, int accumulate,
-                             cudaStream_t s, float *split_buf, size_t cap) {
+                             cudaStream_t s, float *split_buf, size_t cap, double step) {
     using T = PlaneTile<NCH, NP>;
+    // finer rows: more work a view
+    const double share = 1.5 * std::exp2(-8.0 * std::max(0.0, 0.6 - step));
     constexpr size_t smem = T::smem;
     static_assert(smem <= 48 * 1024, "within the default shared-memory limit");
     const dim3 grid((L.n + T::W - 1) / T::W, (L.n + BT_WARPS - 1) / BT_WARPS, (L.n + T::ZT - 1) / T::ZT);
-    return launch_tiles<NCH>(L, a, grid, k_backproject_plane<NCH, NP, ST>, smem, out, accumulate, s, split_buf, cap,
+    return launch_tiles<NCH>(L, a, grid, k_backproject_plane<NCH, NP, ST>, smem, out, accumulate, s, split_buf, cap, share,
                              [&](const BPArgs &b, dim3 g, float *dst, int acc) {
                                  k_backproject_plane<NCH, NP, ST>
                                      <<<g, 32 * BT_WARPS, smem, s>>>(b, L.d_cols_df, L.d_ranges, sino, dst, acc);
@@ -1160,7 +1168,7 @@ int launch_backproject_tilt(const LevelInfo &L, const BPArgs &a, const ST *sino,
                             cudaStream_t s, float *split_buf, size_t cap) {
     using T = TiltTile<NCH>;
     const dim3 grid((L.n + T::W - 1) / T::W, (L.n + BT_WARPS - 1) / BT_WARPS, (L.n + T::ZT - 1) / T::ZT);
-    return launch_tiles<NCH>(L, a, grid, k_backproject_tilt<NCH, ST>, 0, out, accumulate, s, split_buf, cap,
+    return launch_tiles<NCH>(L, a, grid, k_backproject_tilt<NCH, ST>, 0, out, accumulate, s, split_buf, cap, 0.5,
                              [&](const BPArgs &b, dim3 g, float *dst, int acc) {
                                  k_backproject_tilt<NCH, ST><<<g, 32 * BT_WARPS, 0, s>>>(b, L.d_ranges, sino, dst, acc);
                              });
@@ -1172,11 +1180,11 @@ int launch_backproject_tilt(const LevelInfo &L, const BPArgs &a, const ST *sino,
 // more heights.
 template <int NCH, typename ST>
 int launch_backproject_cols(const LevelInfo &L, const BPArgs &a, const ST *sino, float *out, int accumulate,
-                            cudaStream_t s, float *split_buf, size_t cap) {
+                            cudaStream_t s, float *split_buf, size_t cap, double step) {
     constexpr int Z1 = PlaneTile<NCH, 1>::ZT, Z2 = PlaneTile<NCH, 2>::ZT;
     const int t1 = (L.n + Z1 - 1) / Z1 * Z1, t2 = (L.n + Z2 - 1) / Z2 * Z2;
-    if (4 * t2 <= 5 * t1) return launch_backproject_plane<NCH, 2, ST>(L, a, sino, out, accumulate, s, split_buf, cap);
-    return launch_backproject_plane<NCH, 1, ST>(L, a, sino, out, accumulate, s, split_buf, cap);
+    if (4 * t2 <= 5 * t1) return launch_backproject_plane<NCH, 2, ST>(L, a, sino, out, accumulate, s, split_buf, cap, step);
+    return launch_backproject_plane<NCH, 1, ST>(L, a, sino, out, accumulate, s, split_buf, cap, step);
 }
 
 inline BPArgs bp_args(const LevelInfo &L, int view0, int nviews, int stride) {
@@ -1206,7 +1214,8 @@ int launch_backproject(const mgct_geom *g, int level, int view0, int nviews, int
     if constexpr (WEIGHTED && sizeof(ST) == 2) {
         if (g->separable) return launch_backproject16<ST>(L, a, sino, out, accumulate, s, split_buf, cap);
     } else if constexpr (WEIGHTED) {
-        if (g->separable) return launch_backproject_cols<NCH, ST>(L, a, sino, out, accumulate, s, split_buf, cap);
+        if (g->separable)
+            return launch_backproject_cols<NCH, ST>(L, a, sino, out, accumulate, s, split_buf, cap, g->row_step);
         if (columns_padded(g, sizeof(ST))) return launch_backproject_tilt<NCH, ST>(L, a, sino, out, accumulate, s, split_buf, cap);
     }
     if constexpr (!WEIGHTED) {
@@ -1322,7 +1331,7 @@ int launch_backproject_public(const mgct_geom *g, int level, int view0, int nvie
         const int acc = accumulate || c0 ? 1 : 0;
         if (g->separable) {
             MGCT_KERNEL(KK_BACKPROJECT, s, k_weight_rays<ST><<<wgrid, dim3(32, 8), 0, s>>>(a, L.d_cols_df, sc, w));
-            MGCT_TRY((launch_backproject_cols<1, float>(L, a, w, out, acc, s, free_buf, free_cap)));
+            MGCT_TRY((launch_backproject_cols<1, float>(L, a, w, out, acc, s, free_buf, free_cap, g->row_step)));
         } else {
             MGCT_KERNEL(KK_BACKPROJECT, s, k_weight_rays_tilt<ST><<<wgrid, dim3(32, 8), 0, s>>>(a, sc, w));
             MGCT_TRY((launch_backproject_tilt<1, float>(L, a, w, out, acc, s, free_buf, free_cap)));

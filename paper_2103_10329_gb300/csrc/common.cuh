@@ -92,6 +92,7 @@ struct mgct_geom {
     int has_drift;
     int separable;  // 1 if no view has a tilted detector (e_u horizontal, e_v vertical)
     int small_tilt;  // 1 if every view's detector rows lean by at most TILT_MAX from vertical
+    double row_step;  // height step per detector row at the rotation axis, voxels (the same on every grid)
     int levels;
     mgct::LevelInfo lev[8];
     std::vector<mgct::ViewGeom> h_views[8];

@@ -236,6 +236,7 @@ static void e1_range(LevelInfo &L, const std::vector<ViewGeom> &hv) {
 static int upload_tables(mgct_geom *g) {
     int K = g->desc.n_views;
     g->separable = g->small_tilt = 1;
+    g->row_step = g->desc.pixel_pitch * g->desc.n * g->desc.src_axis_dist / g->desc.src_det_dist;
     for (int l = 0; l < g->levels; ++l) {
         auto &hv = g->h_views[l];
         hv.resize(K);
