@@ -148,8 +148,10 @@ int mgct_project(const mgct_geom *geom, int level, int view0, int nviews, int vi
  * major axis) within one voxel of it contributes
  * y * h_g|w|/|w_a| * hat(db) * hat(dc).  Each ray's y * h_g|w|/|w_a| is formed
  * in the handle's quad scratch (in chunks of views) and back-projected plane
- * by plane; with the detector turned by more than 0.35 from upright, or a
- * scratch smaller than one view, a per-voxel gather computes the same sums.
+ * by plane or, for few views and rows much finer or coarser than the voxels,
+ * slab by slab of z; with the detector turned by more than 0.35 from upright,
+ * few turned rays or a scratch smaller than one view, a per-voxel gather
+ * computes the same sums.
  * No atomics: the result is deterministic.  sino: batch sinogram of dtype
  * st; vol_out: float32 [n_g]^3, overwritten (accumulate = 0) or added to
  * (accumulate = 1).  Uses the handle's scratch.

@@ -1094,12 +1094,6 @@ __global__ void k_sum_parts(size_t len, int parts, const float *__restrict__ par
     }
 }
 
-}  // namespace mgct
-
-#include "backproject16.cuh"
-
-namespace mgct {
-
 // Number of view shares for a launch of `blocks` blocks on `sms` multiprocessors
 // that hold `occ` blocks each, at most 16 and `most`: the one with the least
 // estimated time, in units of a view's work on a full chip.  The multiprocessor
@@ -1107,7 +1101,8 @@ namespace mgct {
 // blocks takes 0.4 + 0.45 r / occ; every share writes and reads its partial
 // volumes, `share` views' work: 1.5 in the plane kernel at a row step of 0.6 voxel
 // (public call at 128^3 by 1, 2, 3 shares: 16 views 110, 100, 111 us, 90 views 493,
-// 397, 381; at 200^3, 4 views by 1, 2, 4: 125, 168, 256 us), 0.5 in the tilt kernel.
+// 397, 381; at 200^3, 4 views by 1, 2, 4: 125, 168, 256 us), 0.5 in the tilt kernel,
+// 1 in the slab kernel (one volume a share).
 inline int view_splits(int sms, int occ, int blocks, int nviews, int most, double share) {
     int best = 1;
     double cost = 1e300;
@@ -1122,6 +1117,12 @@ inline int view_splits(int sms, int occ, int blocks, int nviews, int most, doubl
     }
     return best;
 }
+
+}  // namespace mgct
+
+#include "backproject_slab.cuh"
+
+namespace mgct {
 
 // Launches a tile kernel (k_backproject_plane, k_backproject_tilt): both ray
 // classes and the shares of the views in one launch, each into its own partial volume
@@ -1203,20 +1204,22 @@ inline BPArgs bp_args(const LevelInfo &L, int view0, int nviews, int stride) {
 }
 
 // NCH = 2 writes channel c to out + c * n^3.  WEIGHTED: the sinogram carries
-// each ray's dl already (internal solver path) and is stored as
-// weighted_strides says.  split_buf (cap floats, or NULL):
-// scratch for partial volumes.
+// each ray's dl already (internal solver path) and is stored for `route`
+// (weighted_strides).  split_buf (cap floats, or NULL): scratch for partial
+// volumes.
 template <int NCH, typename ST, bool WEIGHTED = false>
 int launch_backproject(const mgct_geom *g, int level, int view0, int nviews, int stride, const ST *sino,
-                       float *out, int accumulate, cudaStream_t s, float *split_buf = nullptr, size_t cap = 0) {
+                       float *out, int accumulate, cudaStream_t s, BpRoute route = BpRoute::GATHER,
+                       float *split_buf = nullptr, size_t cap = 0) {
     const LevelInfo &L = g->lev[level];
     const BPArgs a = bp_args(L, view0, nviews, stride);
-    if constexpr (WEIGHTED && sizeof(ST) == 2) {
-        if (g->separable) return launch_backproject16<ST>(L, a, sino, out, accumulate, s, split_buf, cap);
-    } else if constexpr (WEIGHTED) {
-        if (g->separable)
+    if constexpr (WEIGHTED) {
+        if (route == BpRoute::SLAB) return launch_backproject_slab<NCH, ST>(L, a, sino, out, accumulate, s, split_buf, cap);
+    }
+    if constexpr (WEIGHTED && sizeof(ST) != 2) {
+        if (route == BpRoute::PLANE)
             return launch_backproject_cols<NCH, ST>(L, a, sino, out, accumulate, s, split_buf, cap, g->row_step);
-        if (columns_padded(g, sizeof(ST))) return launch_backproject_tilt<NCH, ST>(L, a, sino, out, accumulate, s, split_buf, cap);
+        if (route == BpRoute::TILT) return launch_backproject_tilt<NCH, ST>(L, a, sino, out, accumulate, s, split_buf, cap);
     }
     if constexpr (!WEIGHTED) {
         if (g->separable) {
@@ -1269,6 +1272,21 @@ __global__ void __launch_bounds__(256)
             w[SINO_PAD + ((size_t)i * a.nu + u0 + r) * pitch + jv] = tile[threadIdx.x][r];
 }
 
+// The same for the slab kernel, to [view][v][u].
+template <typename ST>
+__global__ void k_weight_rows(BPArgs a, const float4 *__restrict__ cols, const ST *__restrict__ sino,
+                              float *__restrict__ w) {
+    const int ju = blockIdx.x * blockDim.x + threadIdx.x;
+    if (ju >= a.nu) return;
+    const int jv = blockIdx.y, i = blockIdx.z;
+    const float4 *c = cols + (size_t)(a.view0 + i * a.stride) * 4 * a.nu + ju;
+    const float rb = __ldg(c).y, ezc = __ldg(c + a.nu).w, e1c = __ldg(c + 2 * a.nu).w;
+    const float rz = fmaf((float)jv - 0.5f * (float)(a.nv - 1), e1c, ezc);
+    const float dl = sqrtf(fmaf(rz, rz, fmaf(rb, rb, 1.0f))) * a.h;
+    const size_t idx = ((size_t)i * a.nv + jv) * a.nu + ju;
+    w[idx] = dl * to_f32(__ldg(sino + idx));
+}
+
 // The same on tilted geometries, each ray's slopes in double-float from the
 // view table.
 template <typename ST>
@@ -1301,11 +1319,10 @@ __global__ void __launch_bounds__(256)
             w[SINO_PAD + ((size_t)i * a.nu + u0 + r) * pitch + jv] = tile[threadIdx.x][r];
 }
 
-// Runs the public A^T through k_weight_rays and the plane kernel (tilted
-// detectors: their own), in chunks of views that fit the quad scratch, and
-// sets *ran; leaves *ran = 0 (nothing launched) where it does not apply:
-// detectors tilted by more than TILT_MAX, no views, or a scratch smaller than
-// one view.
+// Runs the public A^T by weighted rays and the kernel of bp_route, in chunks of
+// views that fit the quad scratch, and sets *ran; leaves *ran = 0 (nothing
+// launched) where it does not apply: the gather's route, no views, or a scratch
+// smaller than one view.
 template <typename ST>
 int launch_backproject_public(const mgct_geom *g, int level, int view0, int nviews, int stride, const ST *sino,
                               float *out, int accumulate, cudaStream_t s, int *ran) {
@@ -1313,8 +1330,11 @@ int launch_backproject_public(const mgct_geom *g, int level, int view0, int nvie
     const LevelInfo &L = g->lev[level];
     const size_t view_elems = (size_t)L.nu * L.nv;
     const size_t cap = 2 * quad_elems(g->lev[0].n) * 4;  // floats in the quad scratch
-    const size_t padded = (size_t)L.nu * (L.nv + SINO_PAD);  // a view of weighted rays
-    if (!columns_padded(g, sizeof(float)) || !L.d_ranges || nviews < 1 || cap < padded + SINO_PAD || L.nv > 65535) return MGCT_OK;
+    if (nviews < 1) return MGCT_OK;
+    const BpRoute route = bp_route(g, L, sizeof(float), nviews, true);
+    const bool slab = route == BpRoute::SLAB;
+    const size_t padded = slab ? view_elems : (size_t)L.nu * (L.nv + SINO_PAD);  // a view of weighted rays
+    if (route == BpRoute::GATHER || !L.d_ranges || cap < padded + SINO_PAD || L.nv > 65535) return MGCT_OK;
     size_t chunk = (cap - SINO_PAD) / padded;
     if (chunk > (size_t)nviews) chunk = nviews;
     if (chunk > 65535) chunk = 65535;
@@ -1329,7 +1349,11 @@ int launch_backproject_public(const mgct_geom *g, int level, int view0, int nvie
         const size_t free_cap = cap > used ? cap - used : 0;
         const ST *sc = sino + (size_t)c0 * view_elems;
         const int acc = accumulate || c0 ? 1 : 0;
-        if (g->separable) {
+        if (slab) {
+            MGCT_KERNEL(KK_BACKPROJECT, s, k_weight_rows<ST><<<dim3((L.nu + 127) / 128, L.nv, cn), 128, 0, s>>>(
+                                               a, L.d_cols_df, sc, w));
+            MGCT_TRY((launch_backproject_slab<1, float>(L, a, w, out, acc, s, free_buf, free_cap)));
+        } else if (route == BpRoute::PLANE) {
             MGCT_KERNEL(KK_BACKPROJECT, s, k_weight_rays<ST><<<wgrid, dim3(32, 8), 0, s>>>(a, L.d_cols_df, sc, w));
             MGCT_TRY((launch_backproject_cols<1, float>(L, a, w, out, acc, s, free_buf, free_cap, g->row_step)));
         } else {

@@ -1,14 +1,15 @@
-// The solver's A^T with 16-bit storage on separable geometries: a thread per
-// voxel column and z slab, in registers (k_backproject_reg) or, for detector
-// rows outside its range of steps, in shared memory (k_backproject_slab).
-// The sinogram is [view][v][u].
+// A^T on separable geometries by a thread per voxel column and z slab, over
+// sinograms stored [view][v][u]: in shared memory (k_backproject_slab) or, for
+// 16-bit storage and detector rows in its range of steps, in registers
+// (k_backproject_reg).  These serve what the plane kernel (backproject.cuh) does
+// not: bp_route in project.cuh has the lines and the figures.
 //
-// float32 storage takes the plane kernel (backproject.cuh), which is faster
-// (865 against 1001 ms per step at 512^3 / 1440 views with BF16 storage) and
-// rounds differently.  16-bit storage keeps these sums bit for bit: the filter
+// 16-bit storage takes them throughout: the plane kernel is faster (865 against
+// 1001 ms per step at 512^3 / 1440 views with BF16 storage) but rounds
+// differently, and 16-bit storage keeps these sums bit for bit -- the filter
 // has no response to a constant, so a step amplifies A^T's rounding about
 // fifty times, and in the next step that moves entries of the 16-bit residual
-// across rounding boundaries -- an iterate changed by 1e-7 differs by 1e-4 one
+// across rounding boundaries: an iterate changed by 1e-7 differs by 1e-4 one
 // step later.
 #pragma once
 
@@ -30,16 +31,29 @@ namespace mgct {
 constexpr int BS_TX = 32, BS_TY = 4, BS_THREADS = BS_TX * BS_TY;
 constexpr float BS_MAGIC = 12582912.0f;  // 1.5 * 2^23
 constexpr int BS_MAGIC_BITS = 0x4B400000;
-// 16 voxels per slab keep the shared slab at 10 KB so that 16 blocks (64
-// warps) fit per SM; guard rows: two below, three above (row pairs reach r + 2)
-constexpr int BS_Z = 16, BS_ROWS = BS_Z + 5;
+template <int NCH>
+struct SlabCfg {
+    // 16 voxels per slab keep the shared slab at 10 KB so that 16 blocks (64
+    // warps) fit per SM; guard rows: two below, three above (row pairs reach r + 2)
+    static constexpr int Z = 16 / NCH, ROWS = Z + 5;
+};
 
+__device__ __forceinline__ float2 load_f2(const float2 *p) { return __ldg(p); }
 template <typename ST>
+__device__ __forceinline__ float2 load_f2(const ST *) { return make_float2(0.0f, 0.0f); }
+
+// DFA = true: 32-bit rays, from the double-float column table; the z crossing is
+// anchored, in double-float, at the detector row nearest the slab's centre, as a
+// whole number of voxels and a rest, and a row's fraction formed from these with
+// the step's low part (vf E1 less whole voxels in one rounding): a weight is
+// accurate to ~1e-7 at any N, as in the plane kernel.  (From one float above the
+// slab: 1e-6; the float32 table's uncentred heights near z = 1000: 6e-5.)
+template <int NCH, typename ST, bool DFA = false>
 __global__ void __launch_bounds__(BS_THREADS)
     k_backproject_slab(BPArgs a, const float4 *__restrict__ cols, const ST *__restrict__ sino,
                        float *__restrict__ out, int accumulate) {
-    constexpr int Z = BS_Z, ROWS = BS_ROWS;
-    __shared__ float acc[ROWS][BS_THREADS];
+    constexpr int Z = SlabCfg<NCH>::Z, ROWS = SlabCfg<NCH>::ROWS;
+    __shared__ float acc[NCH][ROWS][BS_THREADS];
     const int tid = threadIdx.x;
     const int jx = blockIdx.x * BS_TX + (tid % BS_TX), jy = blockIdx.y * BS_TY + tid / BS_TX;
     // blockIdx.z = split * (z-slabs) + slab; split s takes views [i0, i1)
@@ -50,7 +64,9 @@ __global__ void __launch_bounds__(BS_THREADS)
     const int z0 = (blockIdx.z - split * zblocks) * Z;
     const int per = (a.nviews + splits - 1) / splits;
     const int i0 = split * per, i1 = min(a.nviews, i0 + per);
-    for (int r = 0; r < ROWS; ++r) acc[r][tid] = 0.0f;
+#pragma unroll
+    for (int q = 0; q < NCH; ++q)
+        for (int r = 0; r < ROWS; ++r) acc[q][r][tid] = 0.0f;
     if (jx < a.n && jy < a.n) {
         const float ic = 0.5f * (float)(a.n - 1);
         const float cu = 0.5f * (float)(a.nu - 1), cv = 0.5f * (float)(a.nv - 1);
@@ -69,24 +85,59 @@ __global__ void __launch_bounds__(BS_THREADS)
             const int ulo = max(0, (int)ceilf(u0 - hu + cu - 1e-3f));
             const int uhi = min(a.nu - 1, (int)floorf(u0 + hu + cu + 1e-3f));
             const ST *__restrict__ sv = sino + (size_t)i * view_elems;
-            const float4 *__restrict__ ct = cols + (size_t)k * a.nu * 2;
+            const float4 *__restrict__ ct = cols + (size_t)k * a.nu * (DFA ? 4 : 2);
             for (int ju = ulo; ju <= uhi; ++ju) {
-                const float4 t0 = __ldg(ct + 2 * ju);
-                const float4 t1 = __ldg(ct + 2 * ju + 1);
+                const float4 t0 = __ldg(ct + (DFA ? ju : 2 * ju));
+                const float4 t1 = __ldg(ct + (DFA ? a.nu + ju : 2 * ju + 1));
                 const bool ay = t0.x != 0.0f;
                 const float ca = ay ? cy : cx, cb = ay ? cx : cy;
-                const float hb = 1.0f - fabsf(fmaf(ca, t0.y, t0.z) - cb);
-                if (hb <= 0.0f) continue;
-                const float E0 = fmaf(ca, t1.x, t0.w) + ic;  // uncentred z crossing at v' = 0
-                const float E1 = fmaf(ca, t1.z, t1.y);       // its step per row
-                const float rE = __frcp_rn(E1);
-                const float ta = fmaf(zlo - E0, rE, cv), tb = fmaf(zhi - E0, rE, cv);
-                const int vlo = max(0, (int)ceilf(fminf(ta, tb) - 1e-3f));
-                const int vhi = min(a.nv - 1, (int)floorf(fmaxf(ta, tb) + 1e-3f));
-                float vf = (float)vlo - cv;
+                // E0, E1: crossing height at row offset vf = 0 and its slope per
+                // row; zb: the height E0 is counted from (uncentred z)
+                float hb, E0, E1, vf;
+                float E0i = 0.0f, E0f = 0.0f, El = 0.0f;  // DFA: E0 = E0i + E0f, E1's low part
+                int vlo, vhi, zb;
+                if constexpr (!DFA) {
+                    hb = 1.0f - fabsf(fmaf(ca, t0.y, t0.z) - cb);
+                    if (hb <= 0.0f) continue;
+                    E0 = fmaf(ca, t1.x, t0.w) + ic;  // uncentred z crossing at v' = 0
+                    E1 = fmaf(ca, t1.z, t1.y);
+                    const float rE = __frcp_rn(E1);
+                    const float ta = fmaf(zlo - E0, rE, cv), tb = fmaf(zhi - E0, rE, cv);
+                    vlo = max(0, (int)ceilf(fminf(ta, tb) - 1e-3f));
+                    vhi = min(a.nv - 1, (int)floorf(fmaxf(ta, tb) + 1e-3f));
+                    vf = (float)vlo - cv;
+                    zb = z0;
+                } else {
+                    const float4 t2 = __ldg(ct + 2 * a.nu + ju), t3 = __ldg(ct + 3 * a.nu + ju);
+                    const DF eb = df_add(df_mul_f(DF{t0.y, t0.z}, ca), DF{t0.w, t1.x});
+                    hb = 1.0f - fabsf(__fadd_rn(__fsub_rn(eb.hi, cb), eb.lo));
+                    if (hb <= 0.0f) continue;
+                    const DF Eb = df_add(DF{t1.y, t1.z}, df_mul_f(DF{t1.w, t2.x}, ca));  // centred, v' = 0
+                    const DF E1d = df_add(DF{t2.y, t2.z}, df_mul_f(DF{t2.w, t3.x}, ca));
+                    E1 = E1d.hi;
+                    const float zc = (float)z0 - ic + 0.5f * (float)(Z - 1);  // slab centre, centred (exact)
+                    const float va = rintf((zc - Eb.hi) / E1);                // anchor row, centred v'
+                    if (!(fabsf(va) < 1.0e7f)) continue;
+                    const DF c = df_add(df_add(Eb, df_mul_f(E1d, va)), DF{-zc, 0.0f});
+                    E0 = (c.hi + c.lo) + 0.5f * (float)(Z - 1);  // height above z0 at the anchor row
+                    E0i = floorf(E0);
+                    E0f = (c.hi - (E0i - 0.5f * (float)(Z - 1))) + c.lo;
+                    El = E1d.lo;
+                    const float rE = __frcp_rn(E1);
+                    const float ta = fmaf(-1.0f - E0, rE, va + cv), tb = fmaf((float)Z - E0, rE, va + cv);
+                    vlo = max(0, (int)ceilf(fminf(ta, tb) - 1e-3f));
+                    vhi = min(a.nv - 1, (int)floorf(fmaxf(ta, tb) + 1e-3f));
+                    vf = ((float)vlo - cv) - va;  // rows from the anchor (exact)
+                    zb = 0;
+                }
+                // the fraction of a row's height fz above voxel floor(fz)
+                auto frac = [&](float v, float fz, float fl) {
+                    return DFA ? fmaf(v, E1, E0i - fl) + fmaf(v, El, E0f) : fz - fl;
+                };
                 const ST *__restrict__ px = sv + (size_t)vlo * a.nu + ju;
                 int jv = vlo;
-                if (E1 > 0.0f && E1 < 0.999f) {
+                if constexpr (NCH == 1) {
+                  if (E1 > 0.0f && E1 < 0.999f) {
                     // two rows at a time: their crossings floor(fz) are equal or
                     // one apart (0 < E1 < 1), so the pair touches three slab
                     // rows r, r + 1, r + 2 -- three read-modify-writes, not four
@@ -94,43 +145,56 @@ __global__ void __launch_bounds__(BS_THREADS)
                     // (fz + 1.5 * 2^23 holds it in its low mantissa bits); a
                     // row index outside the slab wraps, as unsigned, to the top
                     // guard rows
-                    const int rbase = BS_MAGIC_BITS + z0 - 2;
+                    const int rbase = BS_MAGIC_BITS + zb - 2;
                     for (; jv + 1 <= vhi; jv += 2, vf += 2.0f, px += 2 * (size_t)a.nu) {
                         const float fz0 = fmaf(vf, E1, E0), fz1 = fmaf(vf + 1.0f, E1, E0);
                         const float m0 = __fadd_rd(fz0, BS_MAGIC), m1 = __fadd_rd(fz1, BS_MAGIC);
-                        const float t0 = fz0 - (m0 - BS_MAGIC), t1 = fz1 - (m1 - BS_MAGIC);
+                        const float t0 = frac(vf, fz0, m0 - BS_MAGIC), t1 = frac(vf + 1.0f, fz1, m1 - BS_MAGIC);
                         const int r = (int)min((unsigned)(__float_as_int(m0) - rbase), (unsigned)(ROWS - 3));
                         const bool same = __float_as_int(m1) == __float_as_int(m0);
                         const float y0 = hb * to_f32(__ldg(px)), y1 = hb * to_f32(__ldg(px + a.nu));
                         const float a0 = y0 * t0, b0 = y1 * t1;
                         const float lo1 = y1 - b0;
-                        acc[r][tid] += (y0 - a0) + (same ? lo1 : 0.0f);
-                        acc[r + 1][tid] += a0 + (same ? b0 : lo1);
-                        if (!same) acc[r + 2][tid] += b0;
+                        acc[0][r][tid] += (y0 - a0) + (same ? lo1 : 0.0f);
+                        acc[0][r + 1][tid] += a0 + (same ? b0 : lo1);
+                        if (!same) acc[0][r + 2][tid] += b0;
                     }
+                  }
                 }
                 for (; jv <= vhi; ++jv, vf += 1.0f, px += a.nu) {
                     const float fz = fmaf(vf, E1, E0);
                     const float fl = floorf(fz);
-                    const float t = fz - fl;
+                    const float t = frac(vf, fz, fl);
                     // row of voxel floor(fz) in the guarded slab: in [0, Z + 2]
-                    const int r = min(max((int)fl - z0 + 2, 0), ROWS - 2);
-                    const float yw = hb * to_f32(__ldg(px));
-                    const float w1 = yw * t;
-                    acc[r][tid] += yw - w1;
-                    acc[r + 1][tid] += w1;
+                    const int r = min(max((int)fl - zb + 2, 0), ROWS - 2);
+                    if constexpr (NCH == 1) {
+                        const float yw = hb * to_f32(__ldg(px));
+                        const float w1 = yw * t;
+                        acc[0][r][tid] += yw - w1;
+                        acc[0][r + 1][tid] += w1;
+                    } else {
+                        const float2 y2 = load_f2(px);
+                        const float ya = hb * y2.x, yb = hb * y2.y;
+                        acc[0][r][tid] += ya - ya * t;
+                        acc[0][r + 1][tid] += ya * t;
+                        acc[NCH - 1][r][tid] += yb - yb * t;
+                        acc[NCH - 1][r + 1][tid] += yb * t;
+                    }
                 }
             }
         }
         const size_t nvox = (size_t)a.n * a.n * a.n;
-        float *o = out + (size_t)split * nvox;
+        float *o = out + (size_t)split * NCH * nvox;
         for (int zz = 0; zz < Z; ++zz) {
             const int z = z0 + zz;
             if (z >= a.n) break;
             const size_t idx = ((size_t)z * a.n + jy) * a.n + jx;
-            float v = acc[zz + 2][tid];
-            if (accumulate) v += o[idx];
-            o[idx] = v;
+#pragma unroll
+            for (int q = 0; q < NCH; ++q) {
+                float v = acc[q][zz + 2][tid];
+                if (accumulate) v += o[idx + q * nvox];
+                o[idx + q * nvox] = v;
+            }
         }
     }
 }
@@ -369,23 +433,44 @@ int launch_backproject_reg(const LevelInfo &L, BPArgs a, const ST *sino, float *
     return MGCT_OK;
 }
 
-// A^T of a weighted sinogram stored [view][v][u] (16-bit storage).
-template <typename ST>
-int launch_backproject16(const LevelInfo &L, BPArgs a, const ST *sino, float *out, int accumulate, cudaStream_t s,
-                         float *split_buf, size_t cap) {
-    if (L.e1_lo > BR_E1_LO && L.e1_hi < BR_E1_HI && (size_t)L.nu * (L.nv + 64) < ((size_t)1 << 31))
-        return launch_backproject_reg<ST>(L, a, sino, out, accumulate, s, split_buf, cap);
-    dim3 grid((L.n + BS_TX - 1) / BS_TX, (L.n + BS_TY - 1) / BS_TY, (L.n + BS_Z - 1) / BS_Z);
-    const size_t vol_floats = (size_t)L.n * L.n * L.n;
-    if (split_buf && a.nviews > 1)
-        a.splits = slab_splits(k_backproject_slab<ST>, (int)(grid.x * grid.y * grid.z), a.nviews, vol_floats, cap);
+// A^T of a weighted sinogram stored [view][v][u].
+template <int NCH, typename ST>
+int launch_backproject_slab(const LevelInfo &L, BPArgs a, const ST *sino, float *out, int accumulate, cudaStream_t s,
+                            float *split_buf, size_t cap) {
+    if constexpr (sizeof(ST) == 2) {
+        if (L.e1_lo > BR_E1_LO && L.e1_hi < BR_E1_HI && (size_t)L.nu * (L.nv + 64) < ((size_t)1 << 31))
+            return launch_backproject_reg<ST>(L, a, sino, out, accumulate, s, split_buf, cap);
+    }
+    constexpr int Z = SlabCfg<NCH>::Z;
+    constexpr bool DFA = sizeof(ST) != 2;
+    const float4 *cols = DFA ? L.d_cols_df : L.d_cols;
+    dim3 grid((L.n + BS_TX - 1) / BS_TX, (L.n + BS_TY - 1) / BS_TY, (L.n + Z - 1) / Z);
+    const size_t vol_floats = (size_t)NCH * L.n * L.n * L.n;
+    const int blocks = (int)(grid.x * grid.y * grid.z);
+    if (split_buf && a.nviews > 1) {
+        if constexpr (DFA) {
+            // a share costs one view's work: a partial volume written and read
+            int sms = 0, occ = 0;
+            MGCT_TRY(sm_count(&sms));
+            MGCT_TRY(check_cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                                    &occ, k_backproject_slab<NCH, ST, DFA>, BS_THREADS, 0), "occupancy"));
+            a.splits = view_splits(sms, occ > 0 ? occ : 1, blocks, a.nviews,
+                                   (int)(cap / vol_floats < 64 ? cap / vol_floats : 64), 1.0);
+        } else {
+            a.splits = slab_splits(k_backproject_slab<NCH, ST, DFA>, blocks, a.nviews, vol_floats, cap);
+        }
+    }
     grid.z *= a.splits;
     float *dst = a.splits > 1 ? split_buf : out;
-    MGCT_KERNEL(KK_BACKPROJECT, s,
-                k_backproject_slab<ST><<<grid, BS_THREADS, 0, s>>>(a, L.d_cols, sino, dst, a.splits > 1 ? 0 : accumulate));
+    MGCT_KERNEL(KK_BACKPROJECT, s, k_backproject_slab<NCH, ST, DFA><<<grid, BS_THREADS, 0, s>>>(
+                                       a, cols, sino, dst, a.splits > 1 ? 0 : accumulate));
     if (a.splits > 1) {
         const int sb = (int)((vol_floats + 255) / 256 < 4096 ? (vol_floats + 255) / 256 : 4096);
-        MGCT_KERNEL(KK_BACKPROJECT, s, k_sum_splits<<<sb, 256, 0, s>>>(vol_floats, a.splits, split_buf, out, accumulate));
+        if constexpr (DFA) {
+            MGCT_KERNEL(KK_BACKPROJECT, s, k_sum_parts<<<sb, 256, 0, s>>>(vol_floats, a.splits, split_buf, out, accumulate));
+        } else {
+            MGCT_KERNEL(KK_BACKPROJECT, s, k_sum_splits<<<sb, 256, 0, s>>>(vol_floats, a.splits, split_buf, out, accumulate));
+        }
     }
     return MGCT_OK;
 }

@@ -91,7 +91,7 @@ struct mgct_geom {
     std::vector<double> theta, z, drift;
     int has_drift;
     int separable;  // 1 if no view has a tilted detector (e_u horizontal, e_v vertical)
-    int small_tilt;  // 1 if every view's detector rows lean by at most TILT_MAX from vertical
+    double max_tilt;  // largest lean of a view's detector rows from vertical, |Ev horizontal| / Ev_z
     double row_step;  // height step per detector row at the rotation axis, voxels (the same on every grid)
     int levels;
     mgct::LevelInfo lev[8];

@@ -235,7 +235,8 @@ static void e1_range(LevelInfo &L, const std::vector<ViewGeom> &hv) {
 
 static int upload_tables(mgct_geom *g) {
     int K = g->desc.n_views;
-    g->separable = g->small_tilt = 1;
+    g->separable = 1;
+    g->max_tilt = 0.0;
     g->row_step = g->desc.pixel_pitch * g->desc.n * g->desc.src_axis_dist / g->desc.src_det_dist;
     for (int l = 0; l < g->levels; ++l) {
         auto &hv = g->h_views[l];
@@ -248,7 +249,7 @@ static int upload_tables(mgct_geom *g) {
             if (v.Ev[0] != 0.0f || v.Ev[1] != 0.0f || v.Eu[2] != 0.0f || v.Ev_lo[0] != 0.0f ||
                 v.Ev_lo[1] != 0.0f || v.Eu_lo[2] != 0.0f || v.Q[2] != 0.0f || v.Q[8] != 0.0f)
                 g->separable = 0;
-            if (!(std::hypot((double)v.Ev[0], (double)v.Ev[1]) <= TILT_MAX * (double)v.Ev[2])) g->small_tilt = 0;
+            g->max_tilt = std::max(g->max_tilt, v.Ev[2] > 0.0f ? std::hypot((double)v.Ev[0], (double)v.Ev[1]) / v.Ev[2] : 1e30);
         }
         MGCT_TRY(check_cuda(cudaMemcpy(g->lev[l].d_views, hv.data(), K * sizeof(ViewGeom),
                                        cudaMemcpyHostToDevice),

@@ -16,6 +16,8 @@
 // z) and x-major rays plane x = i of volT [z][x][y] (taps along y, z).
 #pragma once
 
+#include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "common.cuh"
@@ -296,11 +298,51 @@ struct EpiPlus {
     __device__ void finish(double (&)[2]) const {}
 };
 
-// Where element (jv, ju) of view i of a weighted sinogram lies.  In float32
-// and with no or little detector tilt it is [view][u][v], since the
-// back-projector reads down the detector columns (and the column projector's
-// lanes are the rows), with SINO_PAD zero rows before every column and after
-// the last; otherwise [view][v][u].
+// The back-projector of a launch of `views` views with weighted rays of `elem`
+// bytes (4, 8: the two channels of OS-EMTR, 2: 16-bit storage), in the solvers or
+// the public call (`open`).
+//
+// Plane kernel against slab kernel: the slab kernel walks each voxel column's own
+// detector rows; the plane kernel takes 32 heights at a time, needs half the work
+// for each where all have rows (row by row below a step of 0.4 voxel, with tests
+// above 1), and writes at least two volumes and their sum.  So the line is a work,
+// views by heights on the detector, and grows with the distance of the row step
+// from 0.6 to 1 voxel.  It is fitted to 1400 random calls of each kind with either
+// kernel, 8^3 to 288^3, 1 to 120 views, steps of 0.25 to 1.6 and detectors of 1
+// row to 1.9 n; the choice is within 0.6 % (Landweber step), 1 % (OS-EMTR) and 2.5 %
+// (public) of the faster one in the mean.  Slab and plane, us, 128^3 / 192^2: public
+// call 1 view 25 and 29, 4 views 60 and 47, 90 views 1039 and 395; 90 views of step
+// 0.34 1669 and 1829, of step 0.28 and 16 rows 569 and 1210; Landweber step of 8
+// views 253 and 214; OS-EMTR subset of 1 view 160 and 182, of 45 1307 and 859.
+//
+// Tilt kernel against the gather, which sets up every candidate pixel of a voxel:
+// the tilt kernel's columns of steps below 0.5 go ray by ray, a lane at a time, and
+// few rays do not fill its tiles.  Fitted likewise to 600 calls of each kind up to
+// 96^3 (64^3 by the gather and by tiles: 4 views, step 0.41, 0.34 and 0.50 ms; 64
+// views, step 0.69, 3.3 and 0.21 ms; 16^3, 1 view: 21 and 25 us).
+enum class BpRoute { GATHER, SLAB, PLANE, TILT };
+inline BpRoute bp_route(const mgct_geom *g, const LevelInfo &L, size_t elem, int views, bool open) {
+    const double step = g->row_step, n = L.n, H = std::min(n, L.nv * step);  // H: heights on the detector
+    if (!g->separable) {
+        const double least = step * (1.0 - 0.3 * std::min(g->max_tilt, 1.0));
+        const double work = 15.0 * std::exp2(20.0 * std::max(0.0, 0.65 - least) + 2.0 * std::max(0.0, step - 1.2));
+        // the solver's scratch holds shares enough to fill the chip with ray by ray work, too
+        const bool tiny = !open && elem == 4 && n <= 20.0 && views * H >= 70.0;
+        const bool tilt = (views >= 2 || n >= 48.0) && views * H >= work;
+        return elem != 2 && g->max_tilt <= TILT_MAX && (tilt || tiny) ? BpRoute::TILT : BpRoute::GATHER;
+    }
+    const bool small = n <= 36.0;
+    const double base = open ? (small ? 30.0 : 90.0) : elem == 4 ? 200.0 : small ? 90.0 : 450.0;
+    const double work = base * std::exp2((open ? 24.0 : 16.0) * std::max(0.0, 0.6 - step) +
+                                         std::min(4.0, 3.3 * std::max(0.0, step - 1.0)));
+    const bool plane = elem != 2 && views >= (n > 80.0 ? 3 : 2) && views * std::sqrt(H * n) >= work;
+    return plane ? BpRoute::PLANE : BpRoute::SLAB;
+}
+
+// Where element (jv, ju) of view i of a weighted sinogram lies.  For the plane
+// kernels it is [view][u][v], since they read down the detector columns (and
+// the column projector's lanes are the rows), with SINO_PAD zero rows before
+// every column and after the last; otherwise [view][v][u].
 struct SinoStrides {
     int u, v;
     size_t view, first;
@@ -308,13 +350,11 @@ struct SinoStrides {
         return first + (size_t)i * view + (size_t)jv * v + (size_t)ju * u;
     }
 };
-inline bool columns_padded(const mgct_geom *g, size_t elem) {
-    return (g->separable || g->small_tilt) && elem != 2;
-}
-inline SinoStrides weighted_strides(const mgct_geom *g, const LevelInfo &L, size_t elem) {
+inline bool columns_padded(BpRoute r) { return r == BpRoute::PLANE || r == BpRoute::TILT; }
+inline SinoStrides weighted_strides(const LevelInfo &L, BpRoute r) {
     const int pitch = L.nv + SINO_PAD;
-    return columns_padded(g, elem) ? SinoStrides{pitch, 1, (size_t)L.nu * pitch, SINO_PAD}
-                                   : SinoStrides{1, L.nu, (size_t)L.nu * L.nv, 0};
+    return columns_padded(r) ? SinoStrides{pitch, 1, (size_t)L.nu * pitch, SINO_PAD}
+                             : SinoStrides{1, L.nu, (size_t)L.nu * L.nv, 0};
 }
 
 // r = b - A vol and the block's sum of r^2 (float64) into part[block].

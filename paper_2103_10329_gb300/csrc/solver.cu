@@ -188,16 +188,17 @@ static int lw_direction(const mgct_geom *g, int level, const float *mu, const fl
     constexpr bool F32 = std::is_same<ST, float>::value;
     MGCT_TRY(check_cuda(cudaMemsetAsync(w.sums, 0, 8 * sizeof(double), s), "memset"));
     ST *r = reinterpret_cast<ST *>(w.r);
-    if (columns_padded(g, sizeof(ST))) MGCT_TRY(launch_zero_pads((size_t)K * L.nu, L.nv, sizeof(ST), r, s));
+    const BpRoute route = bp_route(g, L, sizeof(ST), K, false);
+    if (columns_padded(route)) MGCT_TRY(launch_zero_pads((size_t)K * L.nu, L.nv, sizeof(ST), r, s));
     int nb = 0;
-    EpiResidual<ST, true> er{r, b, w.part, L.nu, L.nv, K, weighted_strides(g, L, sizeof(ST))};
+    EpiResidual<ST, true> er{r, b, w.part, L.nu, L.nv, K, weighted_strides(L, route)};
     (void)F32;
     MGCT_TRY(project_quads<ST>(g, level, mu, w.muT, w.quads, er, s, &nb));
     (void)nv3;
     MGCT_TRY(launch_sum_partials(w.part, nb, 1, w.sums + 0, s));
     // the quads are free until the line search: room for partial volumes
-    MGCT_TRY(launch_backproject<1, ST, true>(g, level, 0, K, 1, r, w.grad, 0, s, reinterpret_cast<float *>(w.quads),
-                                             2 * quad_elems(L.n) * 4));
+    MGCT_TRY(launch_backproject<1, ST, true>(g, level, 0, K, 1, r, w.grad, 0, s, route,
+                                             reinterpret_cast<float *>(w.quads), 2 * quad_elems(L.n) * 4));
     *d_out = w.grad;
     if (o.precondition) {
         MGCT_TRY(launch_precondition(L.n, g->desc.p_slice_axis, w.grad, w.d, s, g->has_pkernel ? g->pkernel : nullptr));
@@ -215,7 +216,8 @@ static int lw_line_search(const mgct_geom *g, int level, const float *dir, float
     const int K = g->desc.n_views;
     const size_t nv3 = vox(L);
     int nb = 0;
-    EpiDualDot<ST> ed{reinterpret_cast<ST *>(w.r), w.part, L.nu, L.nv, K, weighted_strides(g, L, sizeof(ST))};
+    EpiDualDot<ST> ed{reinterpret_cast<ST *>(w.r), w.part, L.nu, L.nv, K,
+                      weighted_strides(L, bp_route(g, L, sizeof(ST), K, false))};
     MGCT_TRY(project_quads<ST>(g, level, dir, spare, w.quads, ed, s, &nb));
     (void)nv3;
     return launch_sum_partials(w.part, nb, 2, w.sums + slot, s);
@@ -297,14 +299,16 @@ static int osemtr(const mgct_geom *g, int level, int M, float *mu, const float *
     EMSpace w = carve_em(g, level, c);
     const int K = g->desc.n_views;
     const size_t nv3 = vox(L);
-    if (columns_padded(g, sizeof(float2))) MGCT_TRY(launch_zero_pads((size_t)((K + M - 1) / M) * L.nu, L.nv, sizeof(float2), w.c2, s));
+    const int most = (K + M - 1) / M;  // views of the largest subset
+    const BpRoute route = bp_route(g, L, sizeof(float2), most, false);
+    if (columns_padded(route)) MGCT_TRY(launch_zero_pads((size_t)most * L.nu, L.nv, sizeof(float2), w.c2, s));
     for (int m = 0; m < M; ++m) {
         int cnt = (K - m + M - 1) / M;
         if (cnt <= 0) continue;
-        EpiEMTerms e{w.c2, b, pi, L.nu, L.nv, cnt, weighted_strides(g, L, sizeof(float2))};
+        EpiEMTerms e{w.c2, b, pi, L.nu, L.nv, cnt, weighted_strides(L, route)};
         // c2 holds room for every view; past the largest subset's views it is
         // free: room for the column projector's pairs, then for partial volumes
-        const size_t all = padded_sino_elems(K, L.nu, L.nv), used = (padded_sino_elems((K + M - 1) / M, L.nu, L.nv) + 1) & ~(size_t)1;
+        const size_t all = padded_sino_elems(K, L.nu, L.nv), used = (padded_sino_elems(most, L.nu, L.nv) + 1) & ~(size_t)1;
         if (use_column_projector(g, level) && all >= used + 2 * quad_elems(L.n)) {
             int nb = 0;
             MGCT_TRY((project_volume<float, float>(g, level, m, cnt, M, mu, w.muT, w.c2 + used, e, s, &nb)));
@@ -312,7 +316,7 @@ static int osemtr(const mgct_geom *g, int level, int M, float *mu, const float *
             MGCT_TRY(launch_transpose_xy<float>(L.n, mu, w.muT, s));
             MGCT_TRY(launch_project<float>(g, level, m, cnt, M, mu, w.muT, e, s));
         }
-        MGCT_TRY(launch_backproject<2, float2, true>(g, level, m, cnt, M, w.c2, w.nd, 0, s,
+        MGCT_TRY(launch_backproject<2, float2, true>(g, level, m, cnt, M, w.c2, w.nd, 0, s, route,
                                                      reinterpret_cast<float *>(w.c2 + used),
                                                      all > used ? 2 * (all - used) : 0));
         MGCT_TRY(launch_em_update(nv3, mu, w.nd, w.part, s));
