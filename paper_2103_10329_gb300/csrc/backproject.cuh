@@ -20,9 +20,6 @@
 // atomics.
 #pragma once
 
-#include <algorithm>
-#include <cmath>
-
 #include "common.cuh"
 #include "project.cuh"
 
@@ -685,11 +682,13 @@ __global__ void __launch_bounds__(32 * BT_WARPS, PlaneTile<NCH, NP>::MIN_BLOCKS)
 // the anchor row (nearest the tile's middle height), k = Ev_a / w_a and
 // s = r / (1 + k r) = r + d,
 //   z = z_A + s sz,   b = b_A + s sb,
-// where z_A, b_A and the slope sz come from the view table in double-float
-// and d = -k r^2 / (1 + k r) is a small correction: the height above a lane's
-// z keeps its digits (r sz - z in one rounding), a weight is accurate to a few
-// 1e-7.  A lane's first row is the ceiling of the inverse, r = s / (1 - k s),
-// at height z - 1.
+// where z_A, b_A and both slopes come from the view table in double-float and
+// d = -k r^2 / (1 + k r) is a small correction: the height above a lane's z and
+// the distance from a voxel column keep their digits (r sz - z and r sb - j in
+// one rounding, z and j whole numbers), both errors are below 2.5e-7 voxel (5e-8
+// and 3e-8 rms; b as one float from the tile's edge: 1.4e-6 and 3.5e-7).  A
+// lane's first row is the ceiling of the inverse, r = s / (1 - k s), at height
+// z - 1.
 //
 // A height's tent holds at most 4 rows where sz > 1/2, and these fall into at
 // most 3 neighbouring voxel columns where 3 sb < 1: a lane adds 3 sums per
@@ -709,9 +708,10 @@ struct TiltTile {
 struct __align__(16) TiltEntry {
     float sz, szlo;   // height step per row at the anchor
     float d1, rz;     // 1 + height of the anchor row above the tile's middle; 1 / sz
-    float k, sb;      // Ev_a / w_a; step along b per row at the anchor
-    float bA;         // anchor row's b from the tile's edge
-    int jv;           // anchor row
+    float k;          // Ev_a / w_a
+    float sb, sblo;   // sb + sblo: step along b per row at the anchor
+    float bA;         // anchor row's b from the voxel column jA of the tile
+    int jA, jv;       // that column, the nearest; anchor row
     long long base;   // element of the column's row 0
     int i, ju;        // view of the batch and column
 };
@@ -827,10 +827,11 @@ __global__ void __launch_bounds__(32 * BT_WARPS, 3)
             int form = 2;  // 0: 4 rows of one class, 1: 5 rows and a class test, 2: row by row
             TiltEntry t;
             if (ok) {
-                t.i = ib + v * a.splits;
+                const int i = ib + v * a.splits;
+                t.i = i;
                 t.ju = ju;
-                t.base = (long long)SINO_PAD + ((long long)t.i * a.nu + ju) * pitch;
-                const ViewGeom &G = a.views[a.view0 + t.i * a.stride];
+                t.base = (long long)SINO_PAD + ((long long)i * a.nu + ju) * pitch;
+                const ViewGeom &G = a.views[a.view0 + i * a.stride];
                 const float up = (float)ju - cu;
                 const float *N = cls ? G.NY : G.NX, *Nl = cls ? G.NY_lo : G.NX_lo;
                 const int classes = column_classes(G, up, cv);
@@ -852,8 +853,14 @@ __global__ void __launch_bounds__(32 * BT_WARPS, 3)
                 t.rz = 1.0f / sz.hi;
                 t.d1 = __fadd_rn(da.hi, 1.0f) + da.lo;
                 t.k = va.hi * rwa;
-                t.sb = (fmaf(ca, G.Ev[1 - cls], N[2]) - xb.hi * va.hi) * rwa;
-                t.bA = ba.hi + ba.lo;
+                const DF db = df_add(df_add(DF{N[2], Nl[2]}, df_mul_f(DF{G.Ev[1 - cls], G.Ev_lo[1 - cls]}, ca)),
+                                     df_mul(DF{-xb.hi, -xb.lo}, va));
+                const DF sb = df_mul(db, rwa2);
+                t.sb = sb.hi;
+                t.sblo = sb.lo;
+                const float jA = rintf(ba.hi);
+                t.bA = __fsub_rn(ba.hi, jA) + ba.lo;
+                t.jA = (int)jA;
                 t.jv = (int)jf;
                 // over the tile's rows the steps differ from the anchor's by at
                 // most (1 + kr)^2
@@ -865,8 +872,8 @@ __global__ void __launch_bounds__(32 * BT_WARPS, 3)
                 }
                 if (ok && form < 2) {
                     // columns whose rows at the tile's heights all lie off the detector
-                    const float sa = ((float)(-ZT / 2) - t.d1) * t.rz, sb = ((float)(ZT / 2) + 1.0f - t.d1) * t.rz;
-                    const float ra = sa / (1.0f - t.k * sa) + jf, rb = sb / (1.0f - t.k * sb) + jf;
+                    const float s0 = ((float)(-ZT / 2) - t.d1) * t.rz, s1 = ((float)(ZT / 2) + 1.0f - t.d1) * t.rz;
+                    const float ra = s0 / (1.0f - t.k * s0) + jf, rb = s1 / (1.0f - t.k * s1) + jf;
                     ok = ra < (float)a.nv + 1.0f && rb > -2.0f;
                 }
             }
@@ -887,6 +894,7 @@ __global__ void __launch_bounds__(32 * BT_WARPS, 3)
                 const float r0 = __fadd_ru(fmaf(ks * s1, rcp_approx(1.0f - ks), s1), BT_MAGIC) - BT_MAGIC;
                 const int row = (int)r0 + c.jv;
                 const ST *p = sino + c.base + row;
+                const float bA = fmaf(r0, c.sblo, c.bA);  // the low part of the following rows is below 5e-8
                 float w[R], b[R];
                 float2 y[R];
                 // R = 5: the projector's axis choice, ray by ray (ray_dir's own operations)
@@ -904,7 +912,7 @@ __global__ void __launch_bounds__(32 * BT_WARPS, 3)
                     const float r = r0 + (float)s, kr = c.k * r;
                     const float d = -(kr * r) * rcp_approx(1.0f + kr);
                     const float g = fmaf(r, c.sz, -zl) + fmaf(d, c.sz, fmaf(r, c.szlo, c.d1));
-                    b[s] = fmaf(d, c.sb, fmaf(r, c.sb, c.bA));
+                    b[s] = fmaf(d, c.sb, bA);
                     bool in = (unsigned)(row + s) < (unsigned)a.nv;
                     if (R == 5) {
                         const float vp = (float)(row + s) - cv;
@@ -913,17 +921,18 @@ __global__ void __launch_bounds__(32 * BT_WARPS, 3)
                     w[s] = in ? 1.0f - fabsf(g - 1.0f) : -1.0f;
                     y[s] = tl_row(p + s, w[s]);
                 }
-                const float bl = floorf(fminf(b[0], b[R - 1]));
+                // b[s] + (r0 + s) sb: the crossing from voxel column jA
+                const float bl = floorf(fminf(fmaf(r0, c.sb, b[0]), fmaf(r0 + (float)(R - 1), c.sb, b[R - 1])));
                 float2 p0 = both(0.0f), p1 = both(0.0f), p2 = both(0.0f);  // voxel columns bl, bl + 1, bl + 2
 #pragma unroll
                 for (int s = 0; s < R; ++s) {
-                    const float q = b[s] - bl - 1.0f, qm = 1.0f - fabsf(q);  // q in [-1, 1)
+                    const float q = fmaf(r0 + (float)s, c.sb, -1.0f - bl) + b[s], qm = 1.0f - fabsf(q);  // q in [-1, 1)
                     const float2 wy = make_float2(w[s] * y[s].x, NCH == 2 ? w[s] * y[s].y : 0.0f);
                     p1 = fma_f2(both(qm), wy, p1);
                     if (q < 0.0f) p0 = fma_f2(both(-q), wy, p0);
                     if (q > 0.0f) p2 = fma_f2(both(q), wy, p2);
                 }
-                const int j = (int)bl;
+                const int j = (int)bl + c.jA;
                 if ((unsigned)(j + 2) < (unsigned)(W + 2)) {
                     float *d = &accw[0][j + 2][lane];
                     d[0] += p0.x;
