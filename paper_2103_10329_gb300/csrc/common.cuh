@@ -304,8 +304,11 @@ int launch_build_zquads(int n, const SRC *v, void *zy, void *zx, cudaStream_t s)
 // float32 z-fastest pairs, likewise: (V(jz, jb), V(jz, jb + 1))
 template <typename SRC = float>
 int launch_build_zpairs(int n, const SRC *v, void *zy, void *zx, cudaStream_t s);
-// z-fastest lines for the line projector, z padded with zeros to a multiple of
-// 4: v [z][y][x] -> ly [y][x][z] (y-major rays) and lx [x][y][z]
+// z-fastest lines for the line projector, v [z][y][x] -> ly [y][x][z] (y-major
+// rays) and lx [x][y][z].  Lines of a plane: b = -1 .. n at line b + 1 (the outer
+// two are zero), heights 0 .. pitch - 1, zero from n on and in the last four at
+// least.
+__host__ __device__ constexpr int line_pitch(int n) { return ((n + 3) & ~3) + 4; }
 int launch_build_lines(int n, const float *v, float *ly, float *lx, cudaStream_t s);
 template <typename T>
 int launch_transpose_xy(int n, const T *in, T *out, cudaStream_t s);

@@ -3,16 +3,18 @@
 // The projection operator P of Eq. 1 (Sec. 2) is discretised by Joseph's
 // method: each ray is sampled at its crossings with the voxel-centre planes
 // normal to its major axis, by bilinear interpolation within the plane, and
-// each sample carries the path length between planes.  One thread per ray,
-// in two kernels:
-//   k_project_col (tilt-free geometries, the solvers' and mgct_project's
-//     path): a warp takes 32 rows of one detector column, whose rays share
-//     their in-plane crossing, and reads z-fastest copies of the volume;
-//   k_project (any geometry): a warp covers 32 adjacent detector columns of
-//     one detector row, so at every plane its taps fall on one or two
-//     contiguous rows of the volume copy whose fastest axis is the in-plane
-//     horizontal axis.
-// Either way, y-major rays sample plane y = i of vol [z][y][x] (taps along x,
+// each sample carries the path length between planes.  Three kernels:
+//   k_project_lines (tilt-free geometries, float32 volumes from 448 a side): a
+//     block forms the interpolated z line of each of its detector columns once
+//     per plane, and its threads, four rays each, sample these;
+//   k_project_col (other tilt-free calls): a thread per ray, a warp takes 32
+//     rows of one detector column, whose rays share their in-plane crossing,
+//     and reads z-fastest copies of the volume;
+//   k_project (any geometry): a thread per ray, a warp covers 32 adjacent
+//     detector columns of one detector row, so at every plane its taps fall on
+//     one or two contiguous rows of the volume copy whose fastest axis is the
+//     in-plane horizontal axis.
+// In each, y-major rays sample plane y = i of vol [z][y][x] (taps along x,
 // z) and x-major rays plane x = i of volT [z][x][y] (taps along y, z).
 #pragma once
 
@@ -769,9 +771,13 @@ int launch_project(const mgct_geom *g, int level, int view0, int nviews, int str
 // Heights outside the volume are zero in the lines, planes outside a ray's own
 // range therefore sample zero, and no sample is clamped or tested (the clamp
 // of the index only guarantees the bounds).  The heights of a plane's lines
-// run from its first row's crossing to its last row's; where they exceed LP (a
-// detector far coarser than the voxels) the samples are taken from the volume
-// directly.
+// run from its first row's crossing to its last row's, over all its columns;
+// where they exceed LP the samples are taken from the volume directly.  In a
+// block whose columns share a ray class that takes a row step near 1.3 voxels;
+// in one that holds columns of both it happens at any step, since plane pc is
+// then two planes, x = pc and y = pc, crossed at different heights (512^3 /
+// 768^2: up to 215 heights; 1024^3 / 1536^2: 326).  Those are few blocks: the
+// columns around 45 degrees.
 //
 // The copies are plain z-fastest lines [plane][b][z], z padded with zeros to a
 // multiple of 4: 4 bytes a voxel and ray class, half the pairs' footprint.
@@ -785,15 +791,13 @@ int launch_project(const mgct_geom *g, int level, int view0, int nviews, int str
 constexpr int PL_ROWS = 128, PL_COLS = 8, PL_Q = 8, PL_HALF = PL_COLS / 2;
 constexpr int PL_THREADS = 2 * PL_ROWS;
 static_assert(PL_Q == PL_THREADS / 32, "a warp forms one plane's lines");
-// heights a plane's lines may span, and the row step up to which PL_ROWS rows
-// stay within them (with the columns' own spread and margins)
+// heights a plane's lines may span, and the row step up to which PL_ROWS rows of
+// columns of one class stay within them (128 steps of 1.2 are 154; the columns'
+// own spread and the margins take the rest)
 constexpr int PL_LP = 168;
 constexpr float PL_STEP = 1.2f;
 constexpr int PL_WIDE = -0x7fffffff;  // marks a plane beyond that
 
-// Lines of a plane: b = -1 .. n at line b + 1 (the outer two are zero), heights
-// 0 .. pitch - 1, zero from n on and in the last four at least.
-__host__ __device__ constexpr int line_pitch(int n) { return ((n + 3) & ~3) + 4; }
 inline size_t line_elems(int n) { return (size_t)n * (n + 2) * line_pitch(n); }
 
 struct __align__(16) LineTab {

@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(256) k_build_lines(int n, int pitch, const flo
 }
 
 int launch_build_lines(int n, const float *v, float *ly, float *lx, cudaStream_t s) {
-    const int pitch = ((n + 3) & ~3) + 4;  // line_pitch
+    const int pitch = line_pitch(n);
     dim3 grid((pitch + 31) / 32, (n + 31) / 32, n);
     MGCT_KERNEL(KK_TRANSPOSE, s, k_build_lines<<<grid, dim3(32, 8), 0, s>>>(n, pitch, v, ly, lx));
     return MGCT_OK;
