@@ -126,25 +126,25 @@ __global__ void __launch_bounds__(256, 2) k_conv_out(const __nv_bfloat16 *__rest
 }
 
 // Planes a block walks: two of zb + 2 are halo, so as many as leave two blocks
-// for each of the 152 SMs.
-inline int conv_out_planes(int B, int D, int H, int W) {
+// for each multiprocessor.
+inline int conv_out_planes(int sms, int B, int D, int H, int W) {
     const long long tiles = (long long)B * ((H + OL_TY - 1) / OL_TY) * ((W + OL_TX - 1) / OL_TX);
     int zb = OL_ZMAX;
-    while (zb > OL_ZMIN && tiles * ((D + zb - 1) / zb) < 304) zb /= 2;
+    while (zb > OL_ZMIN && tiles * ((D + zb - 1) / zb) < 2LL * sms) zb /= 2;
     return zb;
 }
 
-inline bool conv_out_fits(int B, int D, int H, int W) {  // the grid's y and z limits
-    const int zb = conv_out_planes(B, D, H, W);
+inline bool conv_out_fits(int sms, int B, int D, int H, int W) {  // the grid's y and z limits
+    const int zb = conv_out_planes(sms, B, D, H, W);
     return (H + OL_TY - 1) / OL_TY <= 65535 && (long long)B * ((D + zb - 1) / zb) <= 65535;
 }
 
 // y = conv(in) of the output layer; w [27][wrows][64], row 0 of each tap.
-inline int launch_conv_out(const __nv_bfloat16 *in, const __nv_bfloat16 *w, int wrows, const float *bias, float *out,
-                           int B, int D, int H, int W, cudaStream_t s) {
+inline int launch_conv_out(int sms, const __nv_bfloat16 *in, const __nv_bfloat16 *w, int wrows, const float *bias,
+                           float *out, int B, int D, int H, int W, cudaStream_t s) {
     MGCT_TRY(check_cuda(cudaFuncSetAttribute(k_conv_out, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OL_SMEM),
                         "output layer shared memory"));
-    const int zb = conv_out_planes(B, D, H, W);
+    const int zb = conv_out_planes(sms, B, D, H, W);
     const dim3 grid((W + OL_TX - 1) / OL_TX, (H + OL_TY - 1) / OL_TY, (unsigned)(B * ((D + zb - 1) / zb)));
     MGCT_KERNEL(KK_CONV, s, k_conv_out<<<grid, 256, OL_SMEM, s>>>(in, w, wrows, bias, out, D, H, W, zb));
     return MGCT_OK;

@@ -514,6 +514,8 @@ int mgct_net_create(uint64_t seed, mgct_net **out) {
 // layer by k_conv_out where its grid allows (conv3d_out.cuh).
 static int net_forward(const mgct_net *net, int B, int D, int H, int W, const float *x, const double *ss,
                        double nnorm, const NetSpace &sp, bool inference, cudaStream_t s) {
+    int sms = 0;
+    MGCT_TRY(sm_count(&sms));
     const int nvox = B * D * H * W;
     MGCT_KERNEL(KK_CONV, s, k_net_input<<<std::min((nvox + 255) / 256, 152 * 32), 256, 0, s>>>(x, ss, nnorm, nvox, sp.x0, sp.xs));
     const __nv_bfloat16 *cur = sp.x0;
@@ -528,8 +530,8 @@ static int net_forward(const mgct_net *net, int B, int D, int H, int W, const fl
         a.H = H;
         a.W = W;
         a.nvox = nvox;
-        if (inference && l == NL - 1 && conv_out_fits(B, D, H, W)) {
-            MGCT_TRY(launch_conv_out(cur, net->wf[l], LCOUT[l], net->b[l], sp.y, B, D, H, W, s));
+        if (inference && l == NL - 1 && conv_out_fits(sms, B, D, H, W)) {
+            MGCT_TRY(launch_conv_out(sms, cur, net->wf[l], LCOUT[l], net->b[l], sp.y, B, D, H, W, s));
             break;
         }
         if (l < NL - 1) {
