@@ -781,10 +781,13 @@ int launch_project(const mgct_geom *g, int level, int view0, int nviews, int str
 //
 // The copies are plain z-fastest lines [plane][b][z], z padded with zeros to a
 // multiple of 4: 4 bytes a voxel and ray class, half the pairs' footprint.
-// Profile at 256^3 / 144 views: 73 % L1, 48 % issue-active, waiting for the
-// lines' loads (per sample of a warp 6.3 wavefronts -- lines 3.4, samples 2 --
-// and 16.8 instructions; the column projector 5.8 and 19.5): slower where the
-// pairs stay in L2, faster beyond.  With the next batch's lines held in
+// Profile at 512^3 / 48 middle views: L2 hits a quarter of its reads, 27.7 GB come
+// from DRAM (29 % of its rate; both copies are 1.1 GB), L1 60 %, 41 % issue-active,
+// waiting for the lines' loads: the band of planes that the resident blocks read
+// exceeds L2.  At 256^3 / 144 views, where it does not: 73 % L1, 48 % issue-active
+// (per sample of a warp 6.3 wavefronts -- lines 3.4, samples 2 -- and 16.8
+// instructions; the column projector 5.8 and 19.5), slower than the pairs, which
+// stay in L2.  With the next batch's lines held in
 // registers meanwhile: 23.9 instructions, a third slower at every size; 4
 // planes a batch 10 % slower.
 // ---------------------------------------------------------------------------
@@ -1003,8 +1006,10 @@ __global__ void __launch_bounds__(PL_THREADS, 4)
 // The line projector takes float32 volumes from PL_MIN_N up on tilt-free
 // geometries, to detectors whose rows are at most PL_STEP voxels apart: the
 // pairs' band of planes then no longer fits L2.  Measured per call with its
-// copies (column projector): 1024^3 / 90 views 108 ms (126), 512^3 / 300 views
-// 52.2 (55.3), 256^3 / 720 views 17.3 (15.8), 128^3 / 360 views 1.39 (1.11).
+// copies (column projector): 1024^3 / views 900 to 1079 of 2880 318 ms (378), the
+// first 90 of them, at the volume's face, 108 (122); 512^3 / views 400 to 699 of
+// 1440 70.4 (77.2); 448^3 / views 300 to 499 of 1000 35.4 (34.2), the first 60 9.6
+// (10.0); 256^3 / 720 views 17.3 (15.4); 128^3 / 360 views 1.41 (1.07).
 constexpr int PL_MIN_N = 448;
 inline bool use_line_projector(const mgct_geom *g, int level) {
     const LevelInfo &L = g->lev[level];
