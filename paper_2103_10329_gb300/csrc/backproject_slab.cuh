@@ -4,13 +4,13 @@
 // (k_backproject_reg).  These serve what the plane kernel (backproject.cuh) does
 // not: bp_route in project.cuh has the lines and the figures.
 //
-// 16-bit storage takes them throughout: the plane kernel is faster (865 against
-// 1001 ms per step at 512^3 / 1440 views with BF16 storage) but rounds
-// differently, and 16-bit storage keeps these sums bit for bit -- the filter
-// has no response to a constant, so a step amplifies A^T's rounding about
-// fifty times, and in the next step that moves entries of the 16-bit residual
-// across rounding boundaries: an iterate changed by 1e-7 differs by 1e-4 one
-// step later.
+// 16-bit storage takes them throughout, so far.  The plane kernel is faster there,
+// too (865 against 1001 ms per step at 512^3 / 1440 views with BF16 storage), and
+// more exact, but rounds differently: the filter has no response to a constant,
+// so a step amplifies A^T's rounding about fifty times, and in the next step that
+// moves entries of the 16-bit residual across rounding boundaries -- iterates
+// then differ by up to 2.5e-4 after two steps, the size of 16-bit storage's own
+// error.
 #pragma once
 
 #include "common.cuh"
