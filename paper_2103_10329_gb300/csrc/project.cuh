@@ -476,15 +476,21 @@ struct EpiEMTerms {
 // row (plane 0, corner b = n + 1).  The clamp is exact, not a guard band.
 // ---------------------------------------------------------------------------
 // Plane loads in flight per ray, and resident blocks per SM: 8 and 4, or 4 and 6
-// for pairs in launches of many views of volumes up to 300 a side, whose copies
-// L2 holds whatever runs beside.  Both projections of a Landweber step by views,
-// 8 loads and 4: 128^3 16 views 127 and 129 us, 48 337 and 322, 360 2290 and
-// 2163; 200^3 32 views 0.90 and 0.94 ms, 48 1.28 and 1.24; 256^3 64 views 3.27
-// and 3.39 ms, 128 6.05 and 6.00, 720 32.5 and 31.6; 300^3 128 views 10.7 and
-// 10.8, 240 19.4 and 19.1.  Epilogues that were not faster say so (SMALL_BATCH):
-// a plain residual of 256^3 / 60 views took 1.49 ms with 8 and 2.29 with 4.
+// for pairs of volumes up to 300 a side, whose copies L2 holds whatever runs
+// beside, in launches of many views or of one wave of blocks at 6 and two at 4.
+// Both projections of a Landweber step by views, 8 loads and 4: 128^3 16 views 127
+// and 129 us, 48 337 and 322, 360 2290 and 2163; 200^3 32 views 0.90 and 0.94 ms,
+// 48 1.28 and 1.24; 256^3 64 views 3.27 and 3.39 ms, 128 6.05 and 6.00, 720 32.5
+// and 31.6; 300^3 128 views 10.7 and 10.8, 240 19.4 and 19.1; one wave: 80^3 14
+// views (840 blocks) 55 and 47 us, 64^3 24 views (864) 49 and 44, 10 views of 80^3
+// (600) 39 and 45, 112^3 9 views (1134) 74 and 73.  Epilogues that were not faster
+// say so (SMALL_BATCH): a plain residual of 256^3 / 60 views took 1.49 ms with 8 and
+// 2.29 with 4.
 constexpr int PC_BATCH = 8, PC_BATCH_SMALL = 4;
-inline bool use_small_batch(int n, int nviews) { return n <= 300 && nviews >= 48 && (n <= 200 || nviews >= n); }
+inline bool use_small_batch(int n, int nviews, size_t blocks, int sms) {
+    const double per = (double)blocks / sms;
+    return n <= 300 && ((nviews >= 48 && (n <= 200 || nviews >= n)) || (n <= 200 && per >= 5.1 && per <= 6.7));
+}
 constexpr int PC_TAB = 32;               // planes per table refill (one per lane)
 
 template <typename E>
@@ -715,7 +721,9 @@ int launch_project_col(const mgct_geom *g, int level, int view0, int nviews, int
     if (nblocks) *nblocks = (int)project_blocks_col(L.nu, L.nv, nviews);
     if (nviews == 0) return MGCT_OK;
     if constexpr (LAYOUT == ZL_PAIR && Epi::SMALL_BATCH) {
-        if (use_small_batch(L.n, nviews)) {
+        int sms = 0;
+        MGCT_TRY(sm_count(&sms));
+        if (use_small_batch(L.n, nviews, project_blocks_col(L.nu, L.nv, nviews), sms)) {
             MGCT_KERNEL(KK_PROJECT, s, k_project_col<VT, LAYOUT, PC_BATCH_SMALL, Epi>
                                        <<<grid, dim3(PC_ROWS, PC_COLS), 0, s>>>(a, L.d_cols_df, zqy, zqx, epi));
             return MGCT_OK;
