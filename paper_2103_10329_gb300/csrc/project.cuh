@@ -489,7 +489,7 @@ struct EpiEMTerms {
 constexpr int PC_BATCH = 8, PC_BATCH_SMALL = 4;
 inline bool use_small_batch(int n, int nviews, size_t blocks, int sms) {
     const double per = (double)blocks / sms;
-    return n <= 300 && ((nviews >= 48 && (n <= 200 || nviews >= n)) || (n <= 200 && per >= 5.1 && per <= 6.7));
+    return n <= 300 && ((nviews >= 48 && (n <= 200 || nviews >= n)) || (n <= 200 && per >= 5.1 && per <= 6.8));
 }
 constexpr int PC_TAB = 32;               // planes per table refill (one per lane)
 
